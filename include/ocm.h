@@ -263,12 +263,13 @@ typedef struct ocm_options {
 typedef struct ocm_stats {
     int32_t iterations;     /* improvement sweeps that changed the policy           */
     int32_t cycles;         /* cycles in the final policy graph                     */
-    int32_t detect_rounds;  /* cycle-detection jump rounds, summed over iterations  */
-    int32_t value_rounds;   /* value-propagation jump rounds, summed over iterations */
+    int32_t detect_rounds;  /* one-level evaluations; two-level: rounds on the exits' graph,
+                               summed over iterations                               */
+    int32_t value_rounds;   /* 0 (values are found with the cycles)                 */
     int64_t switched;       /* vertex policy switches summed over iterations        */
     int64_t launches;       /* kernels launched by this call                        */
-    int64_t detect_items;   /* vertex-rounds of work in cycle detection             */
-    int64_t value_items;    /* vertex-rounds of work in value propagation           */
+    int64_t detect_items;   /* vertices evaluated, summed over iterations           */
+    int64_t value_items;    /* 0                                                    */
     int32_t graph_loop;     /* 1: the iteration ran as a CUDA graph, 0: host-driven */
     int32_t rebuild_levels; /* OCM_FLAG_SINGLE_LAMBDA: backward-search levels of the
                                rebuilds, summed over iterations; 0 otherwise         */

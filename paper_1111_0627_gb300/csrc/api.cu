@@ -48,6 +48,7 @@ size_t carve_workspace(void *base, int n, int m, Workspace *ws) {
     w.cyc_rank = static_cast<int *>(take(4 * N));
     w.cid_of_root = static_cast<int *>(take(4 * N));
     w.done = static_cast<unsigned *>(take(4 * ((N + 31) / 32)));
+    w.cyc_tag = static_cast<int *>(take(4 * N));
     w.rec_dirty = static_cast<unsigned *>(take(4 * ((N + 31) / 32)));
     w.scratch16 = static_cast<int4 *>(take(sizeof(int4) * N));
     w.blk_tgt = static_cast<int2 *>(take(sizeof(int2) * ((N + kClassifyBlock - 1) / kClassifyBlock)));
@@ -55,7 +56,6 @@ size_t carve_workspace(void *base, int n, int m, Workspace *ws) {
         take(4 * (((N + kClassifyBlock - 1) / kClassifyBlock + 31) / 32)));
     w.rec_dirty_blk = static_cast<unsigned *>(
         take(4 * (((N + kDirtyBlock - 1) / kDirtyBlock + 31) / 32)));
-    w.sw_iter = static_cast<int *>(take(4 * N));
     w.cls_list = static_cast<int *>(take(4 * N));
     w.cls_hist = static_cast<int *>(take(4 * (size_t)kClassSlots * ((N + kClassifyBlock - 1) / kClassifyBlock)));
     w.band_grp = static_cast<int4 *>(
@@ -79,13 +79,15 @@ size_t carve_workspace(void *base, int n, int m, Workspace *ws) {
     return align_up(off, 256);
 }
 
-__global__ void ctrl_init_kernel(Ctrl *c, long long wait_ns, int frontier, int local_chunks) {
+__global__ void ctrl_init_kernel(Ctrl *c, long long wait_ns, int frontier, int local_chunks,
+                                 int walk_on) {
     Ctrl z;
     memset(&z, 0, sizeof z);
     z.bad_index = INT_MAX;
     z.wait_ns = wait_ns;
     z.frontier = frontier;
     z.local_chunks = local_chunks;
+    z.walk_on = walk_on;
     *c = z;
 }
 
@@ -260,8 +262,37 @@ static int read_ctrl(const Ctrl *dev, Ctrl *host, cudaStream_t st) {
 // termination test, Alg. 1), else advance the iteration index unless the
 // cap is reached.  With use_cond the decision also sets the WHILE node's
 // condition.
-__global__ void loop_control_kernel(Ctrl *c, long long max_iters, int use_cond,
+// It also prepares the counters the next evaluation starts from, and decides
+// whether its record pass marks the records it changes (frontier sweep).
+// One warp: the one-level evaluation's marked cycles that no switch broke stay
+// listed, and their roots are settled for the next evaluation.
+__global__ void loop_control_kernel(Workspace ws, BatchState bs, int n, long long max_iters, int use_cond,
                                     cudaGraphConditionalHandle handle) {
+    Ctrl *c = ws.ctrl;
+    int kept = 0;
+    const bool more = c->err == 0 && c->changed && (long long)c->iter + 1 < max_iters;
+    if (more && ws.walk && c->nrep <= kSettleRoots) {
+        JLS *next = ws.jls[(c->iter + 1) & 1];
+        const int tag = c->iter + 2;   // of the next evaluation
+        const int lane = threadIdx.x;
+        for (int base = 0; base < c->nrep; base += 32) {
+            const int r = base + lane < c->nrep ? ws.cyc_root[base + lane] : -1;
+            const bool keep =
+                r >= 0 && (ws.root_mark[r] & 1) && !(bs.G && bs.gconv[bs.gid[r]]);
+            const unsigned m = __ballot_sync(0xffffffffu, keep);
+            if (keep) {
+                const int pos = kept + __popc(m & ((1u << lane) - 1u));   // (<= base + lane)
+                ws.cyc_root[pos] = r;
+                ws.cid_of_root[r] = pos;
+                ws.root_mark[r] = (tag << 1) | 1;
+                next[r] = JLS{~r, 0, 0};
+            }
+            kept += __popc(m);
+            __syncwarp();
+        }
+    }
+    __syncwarp();
+    if (threadIdx.x) return;
     // the next step's cooperative launches count their barriers from zero
     for (int i = 0; i < 2; ++i) {
         c->bar[i].arrive = 0;
@@ -271,16 +302,25 @@ __global__ void loop_control_kernel(Ctrl *c, long long max_iters, int use_cond,
         }
     }
     c->switched_total += c->switched;
-    int more = 0;
-    if (c->err == 0 && c->changed) {
-        if ((long long)c->iter + 1 >= max_iters) {
-            c->not_converged = 1;
-        } else {
-            c->iter += 1;
-            more = 1;
-        }
+    if (more) c->iter += 1;
+    else if (c->err == 0 && c->changed) c->not_converged = 1;
+    c->mark = c->frontier == 2 ||
+              (c->frontier && (long long)c->switched < ((long long)n >> kFrontierSwitchShift));
+    c->dirty_on = c->mark;
+    c->dirty_cnt = 0;
+    c->changed = 0;
+    c->switched = 0;
+    if (more) {
+        c->nrep = kept;
+        c->old_roots = kept;
     }
-    c->loop_more = more;
+    if (c->walk_on && c->walk_left > (n >> kWalkOffShift)) {
+        c->walk_on = 0;
+        c->walk_fail = 1;
+    }
+    if (!c->walk_on) c->walk_on = !c->walk_fail || c->jump_rounds <= kWalkRounds;
+    c->walk_left = 0;
+    c->loop_more = more ? 1 : 0;
     if (use_cond) cudaGraphSetConditional(handle, more ? 1u : 0u);
 }
 
@@ -323,7 +363,7 @@ static int launch_step(const StepArgs &a, int use_cond, cudaGraphConditionalHand
     if (ks < 0) return -1;
     int k = le + ks;
     if (a.batch) k += launch_batch_converge(a.bs, a.ws, st);
-    loop_control_kernel<<<1, 1, 0, st>>>(a.ws.ctrl, a.max_iters, use_cond, handle);
+    loop_control_kernel<<<1, 32, 0, st>>>(a.ws, a.bs, a.n, a.max_iters, use_cond, handle);
     k += 1;
     if (cudaGetLastError() != cudaSuccess) return -1;
     return k;
@@ -599,7 +639,8 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
                              : (opt->flags & OCM_FLAG_TEST_NO_LOCAL_CHUNKS) ? 0
                              : (opt->flags & OCM_FLAG_TEST_LOCAL_CHUNKS)    ? 2
                                                                            : 1;
-    ctrl_init_kernel<<<1, 1, 0, st>>>(ws.ctrl, wait_ns, frontier, local_chunks);
+    ctrl_init_kernel<<<1, 1, 0, st>>>(ws.ctrl, wait_ns, frontier, local_chunks,
+                                      opt && opt->init_policy ? 1 : 0);
     launch_check_row_ptr(row_ptr, n, m, ws.ctrl, st);
     launches += 2;
     if (bs) launches += launch_batch_prepare(n, m, b, ws, st);
@@ -632,6 +673,9 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
     // pass counts those edges
     const int eval_flags = opt ? opt->flags & (OCM_FLAG_EVAL_LOCAL | OCM_FLAG_EVAL_GLOBAL) : 0;
     const bool local_ok = !bs && !ratio && !single && !(eval_flags & OCM_FLAG_EVAL_GLOBAL);
+    // (the first evaluation's one-step states are written by the initial pass
+    // unless the two-level evaluation is likely)
+    const bool seed = !local_ok || (!(eval_flags & OCM_FLAG_EVAL_LOCAL) && n < kLocalEvalMinN);
     int local_R = 0;
     if (local_ok) {
         const int blocks = evaluate_local_blocks(n);
@@ -642,7 +686,7 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
                        bs ? &b : nullptr, st, local_R,
                        (req_kind == OCM_SWEEP_WINDOW && kind == OCM_SWEEP_CLASSES && !ratio) ? 1
                                                                                             : 0,
-                       band_blocks);
+                       band_blocks, seed ? 1 : 0);
     launches += 3;
     if (cudaGetLastError() != cudaSuccess) return OCM_ERR_CUDA;
     rc = read_ctrl(ws.ctrl, &h, st);
@@ -716,13 +760,18 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
     sa.stall = (opt && (opt->flags & OCM_FLAG_TEST_STALL)) ? 1 : 0;
     sa.N2 = N2;
     sa.max_iters = max_iters;
-    sa.ws = ws;
     sa.bs = b;
     sa.batch = bs != nullptr;
     sa.single = single;
     sa.local = local_ok && ((eval_flags & OCM_FLAG_EVAL_LOCAL) ||
                             (n >= kLocalEvalMinN &&
                              (double)h.local_edges >= kLocalEvalMinFraction * (double)m));
+    ws.walk = sa.local ? 0 : 1;
+    if (ws.walk && !seed) {
+        launch_walk_seed(n, ws, st);
+        launches += 1;
+    }
+    sa.ws = ws;
     sa.no_bitmap = opt && (opt->flags & OCM_FLAG_TEST_NO_BITMAP);
     sa.sg = sg;
     for (int c = 0; c < kClassSlots; ++c) sa.cls_cnt[c] = h.cls_cnt[c];
@@ -756,6 +805,13 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
     if (h.err) return map_err_bits(h.err);
     if (h.not_converged) return OCM_ERR_NOT_CONVERGED;
     const long long it = h.iter;
+    // the one-level evaluation's final states: buffer it & 1 (a batch keeps
+    // the buffer per graph)
+    if (ws.walk && !bs && (it & 1)) {
+        JLS *t = ws.jls[0];
+        ws.jls[0] = ws.jls[1];
+        ws.jls[1] = t;
+    }
 
     phase("ocm:extract");
     // 4. critical cycle(s) of the final policy
@@ -778,7 +834,7 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
         launches += launch_extract(n, Lstar, ws, out.cycle_out, grid, local_R, st);
     }
     if (opt && (opt->eta_num || opt->eta_den || opt->potential || opt->policy)) {
-        launch_outputs(n, ws, opt->eta_num, opt->eta_den, opt->potential, opt->policy, st);
+        launch_outputs(n, ws, b, opt->eta_num, opt->eta_den, opt->potential, opt->policy, st);
         launches += 1;
     }
     if (cudaGetLastError() != cudaSuccess) return OCM_ERR_CUDA;

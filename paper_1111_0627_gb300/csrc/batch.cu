@@ -93,7 +93,7 @@ batch_converge_kernel(BatchState bs, Workspace ws) {
         bs.glen[g] = ws.cyc_L[i];
         bs.gp[g] = ws.cyc_p[i];
         bs.gq[g] = ws.cyc_q[i];
-        bs.gconv[g] = 1;
+        bs.gconv[g] = 1 + (ws.ctrl->iter & 1);   // the buffer of this step's evaluation
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) active += __shfl_xor_sync(0xffffffffu, active, o);
@@ -154,7 +154,7 @@ batch_candidates_kernel(int N, BatchState bs, Workspace ws) {
         bool cand = false;
         if (v < N) {
             const int g = bs.gid[v];
-            const JLS st = ws.jls[0][v];
+            const JLS st = ws.jls[bs.gconv[g] - 1][v];
             cand = (~st.J == bs.groot[g]) && st.len < bs.glen[g];
             if (cand) ws.aprev[v] = v;
         }
@@ -187,7 +187,7 @@ batch_scatter_kernel(BatchState bs, Workspace ws, int32_t *cycle_out) {
         if (ws.aprev[v] == v) {
             const int g = bs.gid[v];
             const int L = bs.glen[g];
-            const int len = ws.jls[0][v].len;
+            const int len = ws.jls[bs.gconv[g] - 1][v].len;
             const int pos = (len == 0) ? 0 : L - len;
             cycle_out[bs.vptr[g] + pos] = ws.pi[v];
             atomicAdd(&bs.gfound[g], 1);

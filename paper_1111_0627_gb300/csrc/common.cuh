@@ -163,7 +163,26 @@ struct Ctrl {
     int chunk_bad;
     int walk_ok;              // extraction: the segment walk found the critical cycle
     long long dirty_cnt;      // how many it changed
+    int mark;                 // the next record pass marks the records it changes
+    // one-level evaluation: whether the vertices walk (0: jump rounds only),
+    // how many walks gave up, and the detection rounds of the last jump phase
+    int walk_on;
+    int walk_left;
+    int old_roots;            // roots listed and settled before the walks
+    int jump_rounds;
+    int walk_fail;            // walks were dropped before in this solve
 };
+
+// One-level evaluation: walks that leave more than n >> kWalkOffShift
+// vertices unresolved are dropped, and every vertex goes to the jump rounds.
+// After that the number of detection rounds of a jump phase tells the depth (r
+// rounds: paths of at most about 2^(r - 1) steps), and the next evaluation
+// walks if it is at most kWalkRounds.  The first evaluation of a cold start
+// jumps: the heaviest edges form a random mapping, about sqrt(n) deep.
+constexpr int kWalkOffShift = 3;
+constexpr int kWalkSteps = 256;
+constexpr int kWalkRounds = 9;
+constexpr int kSettleRoots = 1024;   // roots settled ahead of the walks at most
 
 // The record pass marks the records it changes when the sweep before it
 // switched fewer than n >> kFrontierSwitchShift vertices, and the next sweep
@@ -220,7 +239,8 @@ struct Workspace {
     long long *cyc_key;
     int *cyc_rank;
     int *cid_of_root;
-    unsigned *done;       // bitmap: vertex resolved and its state in both buffers
+    unsigned *done;       // bitmap: extraction scratch
+    int *cyc_tag;         // [n] one-level: tag of the evaluation that marked the cycle v is on (0: none)
     unsigned *rec_dirty;  // bitmap: the last record pass changed v's record (Ctrl::dirty_on)
     unsigned *need_blk;   // bitmap over blocks of kClassifyBlock vertices: some target of
                           //     the block's edges lies in a block with a changed record
@@ -230,7 +250,6 @@ struct Workspace {
     int4 *scratch16;      // [n] two-level evaluation: packed jump states, then node values
                           //     (the records stay intact for the frontier comparison)
     unsigned *rec_dirty_blk;  // bitmap: ... some record of v's block of kDirtyBlock vertices
-    int *sw_iter;         // evaluation index after the sweep that last switched v
     int *cls_list;        // vertices grouped by degree class (stable within a class)
     int *cls_hist;        // per-block class counts, then their exclusive scan
     int4 *band_grp;       // [bands * kClasses + 1] per (band, class), band-major: first
@@ -253,10 +272,47 @@ struct Workspace {
     int *tpi;             // [n] transit time of the policy edge
     long long *jt[2];     // [n] value jumping: transit time of the path from v to J
     long long *recp;      // [n] numerator p of the ratio of v's cycle (gathered by the sweep)
-    int *root_mark;       // [n] two-level evaluation: evaluation stamp of a root found on the node graph
+    int *root_mark;       // [n] one-level: 2 * (tag of the evaluation that listed the root) + 1
+                          //     while its cycle is marked (all its vertices have its cyc_tag,
+                          //     none switched since); two-level evaluation:
+                          //     evaluation stamp of a root found on the node graph
     int2 *chunk_info;     // [n / 1024 + 2] chunked local pass, per block range: (status, exits)
+    // one-level evaluation: jls[k & 1] is the value buffer of evaluation k, and
+    // whatever changes a policy edge stores the vertex's one step {succ, 1,
+    // weight} in the next evaluation's buffer (0 in the two-level form, which
+    // starts from succ and wpi)
+    int walk;
     Ctrl *ctrl;
 };
+
+// v (of the policy just evaluated into buffer F) leaves its policy edge: if it
+// lies on a marked cycle, that cycle is no more.  The vertices of a cycle, its
+// root among them, carry the tag of the evaluation that marked it, so a
+// vertex left over from an earlier cycle has another tag than its root's (or,
+// marked in the same evaluation, unmarks a cycle that still is one, which is
+// then found anew).
+__device__ __forceinline__ void unmark_cycle(const Workspace &ws, int F, int v) {
+    const int t = ws.cyc_tag[v];
+    if (t) {
+        const int root = ~ws.jls[F][v].J;
+        if (root >= 0 && ws.cyc_tag[root] == t) ws.root_mark[root] &= ~1;
+    }
+}
+
+// Policy switch of v for the next evaluation's value buffer (Workspace::walk).
+__device__ __forceinline__ void store_step(const Workspace &ws, int next_eval, int v, int succ,
+                                           int weight) {
+    if (ws.walk) {
+        unmark_cycle(ws, (next_eval ^ 1) & 1, v);
+        ws.jls[next_eval & 1][v] = JLS{succ, 1, (long long)weight};
+    }
+}
+
+// Transit time of a path: below 2^31, under the tag of the evaluation that
+// stored it.
+__device__ __forceinline__ long long path_time(long long tagged) {
+    return tagged & 0xffffffffLL;
+}
 
 // Candidate edge of the improvement sweep and its total order: larger
 // rank(t) first, then larger key q_t * s*w(e) + V(t), then smaller edge index
@@ -305,7 +361,8 @@ struct BatchState {
     int *gfound;                  // [G] cycle vertices found by the extraction
     long long *gp;                // [G] reduced mean of the critical cycle: numerator
     int *gq;                      //     and denominator
-    int *gconv;                   // [G] 1 once the graph's policy is final
+    int *gconv;                   // [G] 0, or 1 + the value buffer (jls[0] or jls[1]) with the
+                                  //     graph's final states once its policy is final
     int *gsw;                     // [G] evaluation index after the last sweep that switched in g
     int *small_queue;             // [G] graphs solved by one block each, largest first
     int G;
@@ -439,7 +496,8 @@ struct NvtxRange {
 void launch_check_row_ptr(const int *row_ptr, int n, int m, Ctrl *ctrl, cudaStream_t st);
 void launch_init_policy(const int *row_ptr, const int *col, const int *w, int sign, int n, int m,
                         const int *init, Workspace ws, const BatchState *bs, cudaStream_t st,
-                        int local_R = 0, int count_win = 0, int band_blocks = 1);
+                        int local_R = 0, int count_win = 0, int band_blocks = 1, int seed = 1);
+void launch_walk_seed(int n, Workspace ws, cudaStream_t st);
 int launch_sweep(const int *row_ptr, const int *col, const int *w, int sign, int n,
                  Workspace ws, const int *cls_cnt, int heavy_edges, BatchState bs, int threads,
                  int band_blocks, cudaStream_t st);
@@ -483,7 +541,7 @@ int launch_csc(const int *row_ptr, const int *col, int n, int m, int *in_ptr, in
 int prepare_connect();
 int launch_connect(const int *row_ptr, const int *col, const int *w, int sign, int n,
                    Workspace ws, SingleWs sw, cudaStream_t st);
-void launch_outputs(int n, Workspace ws, int64_t *eta_num, int32_t *eta_den, int64_t *potential,
+void launch_outputs(int n, Workspace ws, BatchState bs, int64_t *eta_num, int32_t *eta_den, int64_t *potential,
                     int32_t *policy, cudaStream_t st);
 void launch_backward(const int *cycle_edges, int cycle_len, const float *grad_lambda, int m,
                      float *grad_w, cudaStream_t st);

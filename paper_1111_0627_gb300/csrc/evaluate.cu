@@ -31,6 +31,10 @@
 //   materialise: V(v) = q*S(v) - p*len(v), the record {V, rank, q} the next
 //           improvement sweep gathers per edge target.
 //
+// Where the policy graph is shallow, walk_kernel resolves the vertices before
+// this kernel runs, and the jump rounds of detect and values serve what it
+// leaves (see Walks below).
+//
 // Execution: one cooperative launch (all CTAs co-resident) runs every phase;
 // rounds are separated by a grid barrier whose waits are bounded (on expiry
 // the kernel records kErrTimeout and returns).  Rounds are dense over the
@@ -67,6 +71,7 @@ static __device__ __forceinline__ void block_append(int *list, int *s_cnt, bool 
 constexpr int kRankDirectMax = 65536;   // all-pairs rank count up to this many cycles
 constexpr int kRankSplitMin = 4096;     // from this many cycles the count is spread over all blocks
 constexpr int kRankPairTile = 1024;     // keys per piece of the spread count
+constexpr int kTailShared = 1024;       // up to this many cycles every block keeps the table itself
 
 // Inclusive sum of x over the block (all threads call it; 1024 threads).
 static __device__ __forceinline__ int block_inclusive_scan(int x, int *s_warp) {
@@ -233,29 +238,81 @@ static __device__ void evaluate_tail(int n, long long N2, int F, const Workspace
     const int first = blockIdx.x * blockDim.x;
     constexpr bool ratio = RATIO;
     // frontier sweep: mark the records this pass changes?  (decided from the
-    // last sweep's switch count before block 0 clears it below)
-    const int fm = c->frontier;
-    const bool mark = fm != 0 && c->iter > 0 &&
-                      (fm == 2 || (long long)c->switched < ((long long)n >> kFrontierSwitchShift));
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        c->dirty_on = mark ? 1 : 0;
-        c->dirty_cnt = 0;
-    }
-    if (mark && blockIdx.x == 0) {
+    // last sweep's switch count by the loop control kernel)
+    const bool mark = c->mark != 0;
+    if (LOCAL && mark && blockIdx.x == 0) {   // (else the walk kernel clears them)
         const int words = ((n + kDirtyBlock - 1) / kDirtyBlock + 31) / 32;
         for (int i = threadIdx.x; i < words; i += blockDim.x) ws.rec_dirty_blk[i] = 0u;
     }
     // ------------------------------------------------------------ cycles
     // mean W/L, or for the cycle ratio W/T with T the cycle's transit time
     const int K = load_volatile(&c->nrep);
+    // Few cycles (any policy but the first ones): every block computes the
+    // whole cycle table in its own shared memory and no grid barrier is needed
+    // (each of the four below is 1.7 us of an evaluation of 25-80 us); block 0
+    // alone writes the global table.  The walk listed the roots and their
+    // cycle indices before this launch.
+    const bool few = !LOCAL && K <= kTailShared && bs.G == 0;
+    __shared__ long long s_p[LOCAL ? 1 : kTailShared];
+    __shared__ int s_q[LOCAL ? 1 : kTailShared], s_rank[LOCAL ? 1 : kTailShared];
+    __shared__ int s_qmax;
+    if (few) {
+        if (threadIdx.x == 0) s_qmax = 0;
+        __syncthreads();
+        for (int i = threadIdx.x; i < K; i += blockDim.x) {
+            const int root = ws.cyc_root[i];
+            const int x = ws.succ[root];
+            const JLS st = ws.jls[F][x];
+            const long long W = (long long)ws.wpi[root] + st.S;
+            const long long L = 1 + (long long)st.len;
+            const long long Tc = ratio ? (long long)ws.tpi[root] + path_time(ws.jt[F][x]) : L;
+            const long long g = gcd_ll(W, Tc);
+            const long long p = W / g, q = Tc / g;
+            s_p[i] = p;
+            s_q[i] = (int)q;
+            if (ratio) atomicMax(&s_qmax, (int)q);
+            else s_key[i] = mean_key(p, q, N2);
+            if (blockIdx.x == 0) {
+                ws.cyc_p[i] = p;
+                ws.cyc_q[i] = (int)q;
+                ws.cyc_L[i] = (int)L;
+            }
+        }
+        __syncthreads();
+        if (ratio) {
+            // (see below: the keys' bound)
+            const long long qm = s_qmax;
+            const long long N2r = qm * qm;
+            if ((__int128)N2r * (__int128)(c->maxabsw + 1) >= ((__int128)1 << 62)) {
+                if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&c->err, kErrRatioKey);
+                return;
+            }
+            for (int i = threadIdx.x; i < K; i += blockDim.x)
+                s_key[i] = mean_key(s_p[i], s_q[i], N2r);
+            __syncthreads();
+        }
+        for (int i = threadIdx.x; i < K; i += blockDim.x) {
+            const long long key = s_key[i];
+            int rank = 0;
+            for (int j = 0; j < K; ++j) rank += s_key[j] < key;
+            s_rank[i] = rank;
+            if (blockIdx.x == 0) {
+                ws.cyc_rank[i] = rank;
+                atomicMax(&c->best, ((unsigned long long)(unsigned)rank << 32) |
+                                        (unsigned)(INT_MAX - ws.cyc_root[i]));
+            }
+        }
+        __syncthreads();
+    }
     int qmax = 0;
+    if (!few) {
     for (int i = first + threadIdx.x; i < K; i += stride) {
         int root = ws.cyc_root[i];
         int x = ws.succ[root];
         JLS st = LOCAL ? final_value(ws.jls[0], n, x) : ws.jls[F][x];
         long long W = (long long)ws.wpi[root] + st.S;
         long long L = 1 + (long long)st.len;
-        const long long Tc = ratio ? (long long)ws.tpi[root] + ws.jt[F][x] : L;
+        const long long Tc = ratio ? (long long)ws.tpi[root] + path_time(ws.jt[F][x]) : L;
         long long g = gcd_ll(W, Tc);
         long long p = W / g, q = Tc / g;
         ws.cyc_p[i] = p;
@@ -336,12 +393,11 @@ static __device__ void evaluate_tail(int n, long long N2, int F, const Workspace
         if (bs.G) atomicMax(&bs.gbest[bs.gid[root]], packed);
     }
     if (!grid_barrier(c, nblocks)) return;
+    }   // !few
 
     // ------------------------------------------------------- materialise
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        c->changed = 0;
-        c->switched = 0;
-    }
+    const long long *tab_p = few ? s_p : ws.cyc_p;
+    const int *tab_q = few ? s_q : ws.cyc_q, *tab_rank = few ? s_rank : ws.cyc_rank;
     // (warp-uniform trip counts: a warp covers 32 consecutive vertices, one
     // word of the change bitmap, in each of its kMU slots; the slots' loads
     // are issued together, stage by stage)
@@ -376,19 +432,19 @@ static __device__ void evaluate_tail(int n, long long N2, int F, const Workspace
         }
         int ci[kMU];
 #pragma unroll
-        for (int u = 0; u < kMU; ++u) ci[u] = ok[u] ? ws.cid_of_root[~st[u].J] : 0;
+        for (int u = 0; u < kMU; ++u) ci[u] = ok[u] && (LOCAL || K > 1) ? ws.cid_of_root[~st[u].J] : 0;
 #pragma unroll
         for (int u = 0; u < kMU; ++u) {
             const int v = base0 + u * stride + lane;
             bool dirty = false;
             if (ok[u]) {
                 const int i = ci[u];
-                const long long p = ws.cyc_p[i];
-                const int q = ws.cyc_q[i];
+                const long long p = tab_p[i];
+                const int q = tab_q[i];
                 Rec rec;
-                const long long T = ratio ? ws.jt[F][v] : (long long)st[u].len;
+                const long long T = ratio ? path_time(ws.jt[F][v]) : (long long)st[u].len;
                 rec.V = (long long)q * st[u].S - p * T;
-                rec.rank = ws.cyc_rank[i];
+                rec.rank = tab_rank[i];
                 rec.q = q;
                 if (mark) {
                     const Rec old = ws.rec[v];
@@ -446,53 +502,292 @@ static __device__ void evaluate_tail(int n, long long N2, int F, const Workspace
     }
 }
 
-constexpr int kMinMask = 0x7fffffff;
+// ---------------------------------------------------------------------------
+// Walks.  After the first two policies the policy graphs of the random,
+// product and hub graphs are shallow: paths of 10-50 steps to one or a few
+// short cycles, where the jump rounds below cost 14 passes and grid barriers
+// per evaluation.  Instead every vertex walks its policy path, one 16-byte
+// gather a step, adding up (length, weight), until it meets a settled vertex
+// -- one whose state is final, {~root, len, S} -- and settles itself with the
+// sum; no barrier, and every state is read and written by single 128-bit
+// accesses, so a reader sees either the step or the final state.  Both are
+// right, and the final state is the same whatever the order, so results do not
+// depend on the timing.  States are read through L1: all paths share the
+// vertices near the root, and reading those from L2 serialised 10^5 requests
+// on one line (300 us an evaluation); a stale line only costs more steps.
+//   roots: a cycle none of whose vertices switched in the last sweep still is
+// one, with the same root, and its root is settled and listed before the walks
+// start (loop_control_kernel; the sweep clears the cycle's mark when it
+// switches one of its vertices).  Lanes that meet no settled vertex within 32
+// steps may go round a new cycle: one of them looks for it by keeping the
+// vertex passed after 2^k - 1 steps and noticing when it comes back (Brent's
+// cycle finding), settles the cycle's smallest vertex as the root, lists it
+// and marks the cycle's vertices; then they walk again.
+//   passing the root: a walk that passed a new root before it was settled, and
+// met a settled vertex of the cycle after that, has gone round once too often;
+// walks that end at a new root look for its first occurrence.
+//   limit: a warp gives up after kWalkSteps steps or a few new cycles;
+// evaluate_kernel resolves what is left by jump rounds.  While the policy
+// graph is deep (a random first policy has paths of about sqrt(n) steps) the
+// walks are left out altogether: see kWalkRounds.
+//   buffers: evaluation k reads and settles jls[k & 1], where every vertex
+// holds its one step {succ, 1, weight} at the start; a walk writes its own
+// step into the other buffer for evaluation k + 1, where the sweep's switches
+// replace it.
+//   cycle ratio: the path's transit time goes to jt, tagged with the
+// evaluation, before the state is settled; a reader that does not find the
+// tag yet takes the vertex's step instead (no fence, and stale lines of jt are
+// harmless as well).
+// Bound: latency and issue of about 15 gathers a vertex (8 of their sectors
+// from L2); 32 registers keep 64 warps per SM in flight.  Measured per launch
+// with a settled root: 54 us at n = 2.1 M (product graph), 45-50 us at n =
+// 2^20 (random graph), about twice that where a new cycle has to be found.
+// An evaluation (this kernel and the next) against the jump rounds alone,
+// averaged over a solve: 108 against 204 us and 92 against 158 us.  Reading
+// the states past L1 took 220-360 us, and giving each lane its next vertex as
+// soon as it was done (more divergence) 100-300 us.
+// ---------------------------------------------------------------------------
+constexpr int kWalkThreads = 256;
+constexpr int kWalkTight = 32;    // steps between two looks for a cycle
+constexpr int kWalkCycles = 8;    // new cycles a warp looks for
 
-// RATIO: optimal cycle ratio (transit times carried through values and
-// cycles); a separate instance so that the mean keeps its register budget.
+static __device__ __forceinline__ JLS load_state(const JLS *p) {   // (through L1)
+    unsigned long long a, b;
+    asm volatile("{ .reg .b128 t; ld.relaxed.cta.global.b128 t, [%2]; mov.b128 {%0, %1}, t; }"
+                 : "=l"(a), "=l"(b) : "l"(p) : "memory");
+    return JLS{(int)(unsigned)a, (int)(unsigned)(a >> 32), (long long)b};
+}
+
+static __device__ __forceinline__ void store_state(JLS *p, const JLS &s) {
+    const unsigned long long a = (unsigned)s.J | ((unsigned long long)(unsigned)s.len << 32);
+    asm volatile("{ .reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.gpu.global.b128 [%0], t; }"
+                 :: "l"(p), "l"(a), "l"((unsigned long long)s.S) : "memory");
+}
+
+// Looks for a cycle on the path from cur.  Returns its smallest vertex, now
+// settled and listed, or -1 if the path meets a settled vertex or is too long.
+static __device__ __forceinline__ int walk_find_cycle(int cur, JLS *st, unsigned tag,
+                                                   const Workspace &ws) {
+    int tort = cur, lam = 0, power = 1, r = -1;
+    for (int k = 0; k < 2 * kWalkSteps; ++k) {
+        const JLS s = load_state(&st[cur]);
+        if (s.J < 0) return -1;
+        cur = s.J;
+        if (cur == tort) {
+            r = cur;
+            break;
+        }
+        if (++lam == power) {
+            tort = cur;
+            power <<= 1;
+            lam = 0;
+        }
+    }
+    if (r < 0) return -1;
+    int k = 0;
+    for (int y = ws.succ[cur]; y != cur && k < 2 * kWalkSteps; y = ws.succ[y], ++k) r = min(r, y);
+    store_state(&st[r], JLS{~r, 0, 0});
+    // the first to find it lists the root and marks the cycle
+    volatile int *mark = &ws.root_mark[r];
+    if ((unsigned)*mark >> 1 != tag &&
+        (unsigned)atomicExch(&ws.root_mark[r], (int)(tag << 1)) >> 1 != tag) {
+        const int pos = atomicAdd(&ws.ctrl->nrep, 1);
+        ws.cyc_root[pos] = r;
+        ws.cid_of_root[r] = pos;
+        k = 0;
+        int y = r;
+        do {
+            ws.cyc_tag[y] = (int)tag;
+            y = ws.succ[y];
+        } while (y != r && ++k < 2 * kWalkSteps);
+        if (y == r) *mark = (int)(tag << 1) | 1;
+    }
+    return r;
+}
+
 template <bool RATIO>
-__global__ void __launch_bounds__(kEvalThreads, 1)
-evaluate_kernel(int n, long long N2, int max_detect, int max_value, int stall_test, Workspace ws,
-                BatchState bs) {
-    __shared__ long long s_key[kRankTile];
-    __shared__ int s_cnt;
-    grid_sync_start();
+__global__ void __launch_bounds__(kWalkThreads, 8)
+walk_kernel(int n, Workspace ws, BatchState bs) {
     Ctrl *c = ws.ctrl;
-    // vertices whose sw_iter equals this index switched in the last sweep
-    const int eval_index = c->iter;
-    const unsigned nblocks = gridDim.x;
-    const int lane = threadIdx.x & 31;
     const int stride = gridDim.x * blockDim.x;
     const int first = blockIdx.x * blockDim.x;
+    if (c->mark) {   // the frontier sweep's block bits, set by the record pass
+        const int words = ((n + kDirtyBlock - 1) / kDirtyBlock + 31) / 32;
+        for (int i = first + (int)threadIdx.x; i < words; i += stride) ws.rec_dirty_blk[i] = 0u;
+    }
+    if (!c->walk_on) return;
+    const int F = c->iter & 1;
+    const unsigned tag = (unsigned)c->iter + 1u;
+    const int old_roots = c->old_roots;
+    JLS *st = ws.jls[F], *next = ws.jls[F ^ 1];
+    const int lane = threadIdx.x & 31;
+    // settled before the walks (the first entries of the root list; a new
+    // root's cycle index may not be visible yet)
+    auto old_root = [&](int r) -> bool {
+        const int i = ws.cid_of_root[r];
+        return (unsigned)i < (unsigned)old_roots && ws.cyc_root[i] == r;
+    };
+    for (int base = first + (int)threadIdx.x - lane; base < n; base += stride) {
+        const int v = base + lane;
+        const bool on = v < n && !(bs.G && bs.gconv[bs.gid[v]]);
+        JLS s{-1, 0, 0};
+        if (on) {
+            s = load_state(&st[v]);
+            next[v] = s.J >= 0 ? s : JLS{ws.succ[v], 1, (long long)ws.wpi[v]};
+        }
+        int cur = v, len = 0;
+        long long S = 0;
+        unsigned T = 0;          // (n max t < 2^31)
+        int total = 0, found = 0;
+        unsigned open;           // lanes still walking
+        for (;;) {
+#pragma unroll 1
+            for (int k = 0; k < kWalkTight && __any_sync(0xffffffffu, s.J >= 0); ++k) {
+                if (s.J >= 0) {
+                    if (RATIO) T += (unsigned)ws.tpi[cur];
+                    ++len;
+                    S += s.S;
+                    cur = s.J;
+                    s = load_state(&st[cur]);
+                    if (RATIO && s.J < 0 && s.len > 0) {
+                        const long long tt = ws.jt[F][cur];
+                        if ((unsigned)(tt >> 32) == tag)
+                            T += (unsigned)tt;
+                        else   // settled, but its time is not visible yet: one step on
+                            s = JLS{ws.succ[cur], 1, (long long)ws.wpi[cur]};
+                    }
+                }
+            }
+            open = __ballot_sync(0xffffffffu, s.J >= 0);
+            if (!open) break;
+            total += kWalkTight;
+            if (total > kWalkSteps) break;
+            const int leader = __ffs(open) - 1;
+            int r = -1;
+            if (lane == leader) r = walk_find_cycle(cur, st, tag, ws);
+            r = __shfl_sync(0xffffffffu, r, leader);
+            if (r >= 0) {
+                if (++found > kWalkCycles) break;
+                if (s.J >= 0) {   // from the start, the root being settled now
+                    cur = v;
+                    len = 0;
+                    S = 0;
+                    T = 0;
+                    s = load_state(&st[v]);
+                }
+            }
+        }
+        if (on && s.J < 0) {
+            const int root = ~s.J;
+            JLS f{s.J, len + s.len, S + s.S};
+            if (root == v) {
+                f = JLS{~v, 0, 0};
+                T = 0;
+            } else if (!old_root(root)) {   // a new root: passed on the way?
+                int y = v, k = 0;
+                while (k < len && y != root) {
+                    y = ws.succ[y];
+                    ++k;
+                }
+                if (k < len) {
+                    f = JLS{~root, k, 0};
+                    T = 0;
+                    for (y = v; y != root; y = ws.succ[y]) {   // (k steps)
+                        f.S += ws.wpi[y];
+                        if (RATIO) T += (unsigned)ws.tpi[y];
+                    }
+                }
+            }
+            if (RATIO) ws.jt[F][v] = ((long long)tag << 32) | T;
+            store_state(&st[v], f);
+        }
+        if (open) {
+            int sofar = 0;
+            if (lane == 0) sofar = atomicAdd(&c->walk_left, __popc(open));
+            sofar = __shfl_sync(0xffffffffu, sofar, 0);
+            if (sofar > (n >> kWalkOffShift)) return;   // (evaluate_kernel resolves everything)
+        }
+    }
+}
+
+// The first evaluation's one-step states (when the initial pass left them out).
+__global__ void __launch_bounds__(kThreads) walk_seed_kernel(int n, Workspace ws) {
+    const int stride = gridDim.x * blockDim.x;
+    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+        ws.jls[0][v] = JLS{ws.succ[v], 1, (long long)ws.wpi[v]};
+        ws.cyc_tag[v] = 0;
+    }
+}
+
+void launch_walk_seed(int n, Workspace ws, cudaStream_t st) {
+    int blocks = (n + kThreads - 1) / kThreads;
+    if (blocks > 4096) blocks = 4096;
+    prof_begin(kProfInit, st);
+    walk_seed_kernel<<<blocks, kThreads, 0, st>>>(n, ws);
+    prof_end(kProfInit, st);
+}
+
+// Jump rounds over the vertices the walks left (all of them once the walks
+// are off): detection by window minima, then values, as described at the top
+// of the file; every final state ends in jls[F] (times in jt[F]).  Scratch:
+// the 16-byte scratch is the other value buffer.  Returns false on an error or
+// when a grid barrier gave up (recorded in the control block).
+template <bool RATIO>
+static __device__ bool jump_resolve(int n, int F, bool all, int max_detect, int max_value,
+                                    const Workspace &ws, const BatchState &bs, int *s_cnt) {
+    Ctrl *c = ws.ctrl;
+    constexpr bool ratio = RATIO;   // optimal cycle ratio: times ride along
+    const unsigned nblocks = gridDim.x;
+    const int lane = threadIdx.x & 31;
     // every block owns a contiguous vertex range and keeps its worklist of
     // unfinished vertices inside the same range of the two list buffers
     const int R = (n + (int)gridDim.x - 1) / (int)gridDim.x;
     const int lo = min((int)blockIdx.x * R, n), hi = min(lo + R, n);
     int *LA = ws.list[0] + lo, *LB = ws.list[1] + lo;
-
-    constexpr bool ratio = RATIO;   // optimal cycle ratio: times ride along
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        c->nrep = 0;
-        c->best = 0;
-        c->qmax = 0;
-    }
-    for (int g = first + threadIdx.x; g < bs.G; g += stride) bs.gbest[g] = 0;
-    if (threadIdx.x == 0) s_cnt = 0;
-    // No grid barrier is needed here: the counters reset above are first
-    // used after the barrier that ends detection round 0 (round 0 resolves
-    // nothing), and gbest only at the end.
+    JLS *V[2] = {ws.jls[F], reinterpret_cast<JLS *>(ws.scratch16)};
+    long long *VT[2] = {ws.jt[F], ws.jt[F ^ 1]};
+    if (threadIdx.x == 0) *s_cnt = 0;
     __syncthreads();
-    // (test only: wait for one block more than exists, so the wait expires)
-    if (stall_test && !grid_barrier(c, nblocks + 1u)) return;
+    // ---- the worklist; settled vertices are resolved in both buffers
+    for (int i0 = 0; i0 < hi - lo; i0 += blockDim.x) {
+        const int i = i0 + threadIdx.x;
+        const int v = lo + i;
+        bool keep = false;
+        // batched: vertices of converged graphs keep everything
+        if (i < hi - lo && !(bs.G && bs.gconv[bs.gid[v]])) {
+            const JLS s = all ? JLS{0, 0, 0} : V[0][v];
+            if (s.J >= 0) {
+                keep = true;
+                // (no walk wrote the next evaluation's step)
+                if (all) ws.jls[F ^ 1][v] = JLS{ws.succ[v], 1, (long long)ws.wpi[v]};
+            } else {
+                const JM f{s.J, 0};
+                ws.jm[0][v] = f;
+                ws.jm[1][v] = f;
+                ws.rep[v] = ~s.J;
+                V[1][v] = s;
+                if (ratio) VT[0][v] = VT[1][v] = path_time(VT[0][v]);
+            }
+        }
+        block_append(LA, s_cnt, keep, v, lane);
+    }
+    __syncthreads();
+    const int cnt0 = *s_cnt;
+    __syncthreads();
+    if (threadIdx.x == 0) *s_cnt = 0;
+    // (the list of unfinished vertices is needed again for the values)
+    int *LC = ws.list[2] + lo;
+    for (int i = threadIdx.x; i < cnt0; i += blockDim.x) {
+        const int v = LA[i];
+        LC[i] = v;
+        ws.jm[0][v] = JM{ws.succ[v], v};
+    }
+    if (!grid_barrier(c, nblocks)) return false;
 
     // ------------------------------------------------------------ detect
-    // State: unresolved {J >= 0, M | dirty << 31}; resolved {~root, dirty}.
-    // "dirty" ORs, over the same windows as M, whether a vertex switched in
-    // the sweep before this evaluation; at resolution it covers v's whole
-    // path and cycle, so a clean vertex keeps last evaluation's path sums.
-    int cnt = hi - lo;
-    int r = 0;
-    for (;; ++r) {
+    // State: unresolved {J >= 0, window minimum}; resolved {~root, 0}.
+    int cnt = cnt0;
+    for (int r = 0;; ++r) {
         const JM *in = ws.jm[r & 1];
         JM *out = ws.jm[(r + 1) & 1];
         int *lin = (r & 1) ? LB : LA;
@@ -505,34 +800,19 @@ evaluate_kernel(int n, long long N2, int max_detect, int max_value, int stall_te
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
                 const int i = i0 + u * blockDim.x + threadIdx.x;
-                item[u] = INT_MIN;
-                if (i < cnt) {
-                    item[u] = (r == 0) ? lo + i : lin[i];
-                    // batched: vertices of converged graphs keep everything
-                    if (r == 0 && bs.G && bs.gconv[bs.gid[lo + i]]) item[u] = INT_MIN;
-                }
+                item[u] = i < cnt ? lin[i] : INT_MIN;
             }
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
                 const int it = item[u];
                 if (it == INT_MIN) continue;
                 const int v = it < 0 ? ~it : it;
-                if (r == 0) {
-                    s[u] = JM{ws.succ[v], v | ((ws.sw_iter[v] == eval_index) ? INT_MIN : 0)};
-                    ap[u] = -1;
-                } else {
-                    s[u] = in[v];
-                    ap[u] = it >= 0 ? ws.aprev[v] : 0;
-                }
+                s[u] = in[v];
+                ap[u] = (r > 0 && it >= 0) ? ws.aprev[v] : -1;
             }
 #pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                const int it = item[u];
-                if (it == INT_MIN || it < 0) continue;
-                const int J = s[u].J;
-                t[u] = (r == 0) ? JM{ws.succ[J], J | ((ws.sw_iter[J] == eval_index) ? INT_MIN : 0)}
-                                : in[J];
-            }
+            for (int u = 0; u < kU; ++u)
+                if (item[u] != INT_MIN && item[u] >= 0) t[u] = in[s[u].J];
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
                 const int it = item[u];
@@ -543,23 +823,19 @@ evaluate_kernel(int n, long long N2, int max_detect, int max_value, int stall_te
                     if (it < 0) {
                         out[v] = s[u];        // resolved last round: copy forward
                     } else {
-                        const int sdirty = (int)((unsigned)s[u].M >> 31);
-                        int root = -1, dirty = 0;
+                        int root = -1;
                         if (t[u].J < 0) {
                             root = ~t[u].J;   // target resolved: it lies on v's path
-                            dirty = sdirty | t[u].M;
-                        } else if (r > 0 && (t[u].M & kMinMask) == ap[u]) {
+                        } else if (r > 0 && t[u].M == ap[u]) {
                             root = ap[u];     // smallest vertex of the cycle
-                            dirty = sdirty | (int)((unsigned)t[u].M >> 31);
                         } else {
                             // (round 0: J_0 = succ, M_0(v) = v, no test yet)
-                            const int m = min(s[u].M & kMinMask, t[u].M & kMinMask);
-                            out[v] = JM{t[u].J, m | ((s[u].M | t[u].M) & INT_MIN)};
-                            ws.aprev[v] = t[u].M & kMinMask;
+                            out[v] = JM{t[u].J, min(s[u].M, t[u].M)};
+                            ws.aprev[v] = t[u].M;
                             keep = true;
                         }
                         if (root >= 0) {
-                            out[v] = JM{~root, dirty};
+                            out[v] = JM{~root, 0};
                             ws.rep[v] = root;
                             resolved = true;
                             is_root = (root == v);
@@ -567,182 +843,218 @@ evaluate_kernel(int n, long long N2, int max_detect, int max_value, int stall_te
                         ++pend;
                     }
                 }
-                block_append(lout, &s_cnt, keep || resolved, keep ? v : ~v, lane);
+                block_append(lout, s_cnt, keep || resolved, keep ? v : ~v, lane);
                 kept += keep;
                 const int pos = warp_append(&c->nrep, is_root, lane);
-                if (is_root) ws.cyc_root[pos] = v;
+                if (is_root) {
+                    ws.cyc_root[pos] = v;
+                    ws.cid_of_root[v] = pos;
+                }
             }
         }
         __syncthreads();
-        cnt = s_cnt;
+        cnt = *s_cnt;
         __syncthreads();
-        if (threadIdx.x == 0) s_cnt = 0;
+        if (threadIdx.x == 0) *s_cnt = 0;
         bool ok;
         int still;   // vertices still unresolved after this round
         const int left = grid_sum2_barrier(c, nblocks, pend, kept, &still, &ok);
-        if (!ok) return;
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            c->rounds_detect += 1;
-            c->items_detect += left;
-        }
-        if (left == 0) break;
-        if (still == 0) {
-            // all resolved: instead of a round that only copies the states
-            // resolved in this one into the other buffer, each block copies
-            // its own (the list it just built) -- nothing reads another
-            // block's jump state before the kernel ends
-            for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-                const int v = ~lout[i];
-                ws.jm[r & 1][v] = out[v];
-            }
-            __syncthreads();
+        if (!ok) return false;
+        if (left == 0 || still == 0) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) c->jump_rounds = r + 1;
             break;
         }
         if (r + 1 >= max_detect) {
             if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&c->err, kErrDetect);
-            return;
+            return false;
         }
     }
 
     // ------------------------------------------------------------ values
-    // Only dirty vertices are recomputed: a clean vertex's path and cycle are
-    // those of the last evaluation, whose final (root, len, S) is still in
-    // both buffers.  Dirty roots are final at once, as is a dirty vertex whose
-    // successor is a root; the rest jump until they meet a final state.
+    // Roots are final at once, as is a vertex whose successor is a root; the
+    // rest jump until they meet a final state.
     cnt = 0;
     int left0 = 0;
     {
         int pend = 0;
-        for (int i0 = 0; i0 < hi - lo; i0 += blockDim.x) {
+        for (int i0 = 0; i0 < cnt0; i0 += blockDim.x) {
             const int i = i0 + threadIdx.x;
             bool keep = false;
-            int v = lo + i;
-            if (i < hi - lo && !(bs.G && bs.gconv[bs.gid[v]])) {
-                const JM d = ws.jm[0][v];
-                if (d.M) {
-                    const int root = ~d.J;
-                    JLS st;
-                    long long T = 0;
-                    bool fin = true;
-                    if (root == v) {
-                        st = JLS{~v, 0, 0};
-                    } else {
-                        const int sv = ws.succ[v];
-                        fin = (ws.rep[sv] == sv);
-                        st = JLS{fin ? ~sv : sv, 1, (long long)ws.wpi[v]};
-                        if (ratio) T = ws.tpi[v];
-                    }
-                    ws.jls[0][v] = st;
-                    if (fin) ws.jls[1][v] = st;
-                    if (ratio) {
-                        ws.jt[0][v] = T;
-                        if (fin) ws.jt[1][v] = T;
-                    }
-                    keep = !fin;
+            int v = 0;
+            if (i < cnt0) {
+                v = LC[i];
+                const int root = ws.rep[v];
+                JLS st;
+                long long T = 0;
+                bool fin = true;
+                if (root == v) {
+                    st = JLS{~v, 0, 0};
+                } else {
+                    const int sv = ws.succ[v];
+                    fin = (ws.rep[sv] == sv);
+                    st = JLS{fin ? ~sv : sv, 1, (long long)ws.wpi[v]};
+                    if (ratio) T = ws.tpi[v];
                 }
+                V[0][v] = st;
+                if (fin) V[1][v] = st;
+                if (ratio) {
+                    VT[0][v] = T;
+                    if (fin) VT[1][v] = T;
+                }
+                keep = !fin;
             }
-            block_append(LA, &s_cnt, keep, v, lane);
+            block_append(LA, s_cnt, keep, v, lane);
             pend += keep;
         }
         __syncthreads();
-        cnt = s_cnt;
+        cnt = *s_cnt;
         __syncthreads();
-        if (threadIdx.x == 0) s_cnt = 0;
+        if (threadIdx.x == 0) *s_cnt = 0;
         bool ok;
         left0 = grid_sum_barrier(c, nblocks, pend, &ok);
-        if (!ok) return;
+        if (!ok) return false;
     }
-    int F = 0;   // a value buffer holding every final state (both, once copied forward)
-    if (left0 != 0) {
-        for (int j = 1;; ++j) {
-            const JLS *in = ws.jls[(j + 1) & 1];
-            JLS *out = ws.jls[j & 1];
-            // cycle ratio: the transit time of the path to J, jumped alongside
-            const long long *tin = ws.jt[(j + 1) & 1];
-            long long *tout = ws.jt[j & 1];
-            int *lin = (j & 1) ? LA : LB;
-            int *lout = (j & 1) ? LB : LA;
-            int pend = 0, kept = 0;
-            for (int i0 = 0; i0 < cnt; i0 += kU * blockDim.x) {
-                int item[kU];
-                JLS s[kU], t[kU];
-                long long ts[kU], tt[kU];
+    if (left0 == 0) return true;
+    for (int j = 1;; ++j) {
+        const JLS *in = V[(j + 1) & 1];
+        JLS *out = V[j & 1];
+        // cycle ratio: the transit time of the path to J, jumped alongside
+        const long long *tin = VT[(j + 1) & 1];
+        long long *tout = VT[j & 1];
+        int *lin = (j & 1) ? LA : LB;
+        int *lout = (j & 1) ? LB : LA;
+        int pend = 0, kept = 0;
+        for (int i0 = 0; i0 < cnt; i0 += kU * blockDim.x) {
+            int item[kU];
+            JLS s[kU], t[kU];
+            long long ts[kU], tt[kU];
 #pragma unroll
-                for (int u = 0; u < kU; ++u) {
-                    const int i = i0 + u * blockDim.x + threadIdx.x;
-                    item[u] = i < cnt ? lin[i] : INT_MIN;
-                }
+            for (int u = 0; u < kU; ++u) {
+                const int i = i0 + u * blockDim.x + threadIdx.x;
+                item[u] = i < cnt ? lin[i] : INT_MIN;
+            }
 #pragma unroll
-                for (int u = 0; u < kU; ++u) {
-                    const int it = item[u];
-                    if (it != INT_MIN) {
-                        s[u] = in[it < 0 ? ~it : it];
-                        if (ratio) ts[u] = tin[it < 0 ? ~it : it];
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < kU; ++u)
-                    if (item[u] != INT_MIN && item[u] >= 0) {
-                        t[u] = in[s[u].J];
-                        if (ratio) tt[u] = tin[s[u].J];
-                    }
-#pragma unroll
-                for (int u = 0; u < kU; ++u) {
-                    const int it = item[u];
-                    bool keep = false, fin = false;
-                    int v = 0;
-                    if (it != INT_MIN) {
-                        v = it < 0 ? ~it : it;
-                        if (it < 0) {
-                            out[v] = s[u];    // final last round: copy forward
-                            if (ratio) tout[v] = ts[u];
-                        } else {
-                            const JLS nu{t[u].J, s[u].len + t[u].len, s[u].S + t[u].S};
-                            out[v] = nu;
-                            if (ratio) tout[v] = ts[u] + tt[u];
-                            fin = nu.J < 0;
-                            keep = !fin;
-                            ++pend;
-                        }
-                    }
-                    block_append(lout, &s_cnt, keep || fin, keep ? v : ~v, lane);
-                    kept += keep;
+            for (int u = 0; u < kU; ++u) {
+                const int it = item[u];
+                if (it != INT_MIN) {
+                    s[u] = in[it < 0 ? ~it : it];
+                    if (ratio) ts[u] = tin[it < 0 ? ~it : it];
                 }
             }
-            __syncthreads();
-            cnt = s_cnt;
-            __syncthreads();
-            if (threadIdx.x == 0) s_cnt = 0;
-            bool ok;
-            int still;
-            const int left = grid_sum2_barrier(c, nblocks, pend, kept, &still, &ok);
-            if (!ok) return;
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
-                c->rounds_value += 1;
-                c->items_value += left;
-            }
-            if (left == 0) break;
-            if (still == 0) {
-                // all final: the phases below read buffer F, which holds
-                // every final state; each block copies the states its
-                // vertices reached in this round into the other buffer
-                // (read by no one before the kernel ends)
-                F = j & 1;
-                for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-                    const int v = ~lout[i];
-                    ws.jls[(j + 1) & 1][v] = out[v];
-                    if (ratio) ws.jt[(j + 1) & 1][v] = tout[v];
+#pragma unroll
+            for (int u = 0; u < kU; ++u)
+                if (item[u] != INT_MIN && item[u] >= 0) {
+                    t[u] = in[s[u].J];
+                    if (ratio) tt[u] = tin[s[u].J];
                 }
-                break;
-            }
-            if (j + 1 > max_value) {
-                if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&c->err, kErrValue);
-                return;
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int it = item[u];
+                bool keep = false, fin = false;
+                int v = 0;
+                if (it != INT_MIN) {
+                    v = it < 0 ? ~it : it;
+                    if (it < 0) {
+                        out[v] = s[u];    // final last round: copy forward
+                        if (ratio) tout[v] = ts[u];
+                    } else {
+                        const JLS nu{t[u].J, s[u].len + t[u].len, s[u].S + t[u].S};
+                        out[v] = nu;
+                        if (ratio) tout[v] = ts[u] + tt[u];
+                        fin = nu.J < 0;
+                        keep = !fin;
+                        ++pend;
+                    }
+                }
+                block_append(lout, s_cnt, keep || fin, keep ? v : ~v, lane);
+                kept += keep;
             }
         }
+        __syncthreads();
+        cnt = *s_cnt;
+        __syncthreads();
+        if (threadIdx.x == 0) *s_cnt = 0;
+        bool ok;
+        int still;
+        const int left = grid_sum2_barrier(c, nblocks, pend, kept, &still, &ok);
+        if (!ok) return false;
+        if (left == 0) break;
+        if (still == 0) {
+            // all final: the phases that follow read buffer 0; the states
+            // reached in this round go there too
+            if (j & 1) {
+                for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
+                    const int v = ~lout[i];
+                    V[0][v] = out[v];
+                    if (ratio) VT[0][v] = tout[v];
+                }
+                if (!grid_barrier(c, nblocks)) return false;
+            }
+            break;
+        }
+        if (j + 1 > max_value) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&c->err, kErrValue);
+            return false;
+        }
     }
+    return true;
+}
 
+// RATIO: optimal cycle ratio (transit times carried through values and
+// cycles); a separate instance so that the mean keeps its register budget.
+template <bool RATIO>
+__global__ void __launch_bounds__(kEvalThreads, 1)
+evaluate_kernel(int n, long long N2, int max_detect, int max_value, int stall_test, Workspace ws,
+                BatchState bs) {
+    __shared__ long long s_key[kRankTile];
+    __shared__ int s_cnt;
+    grid_sync_start();
+    Ctrl *c = ws.ctrl;
+    const unsigned nblocks = gridDim.x;
+    const int F = c->iter & 1;   // the value buffer of this evaluation
+    const int left = c->walk_left;
+    // (walks that were cut short may have settled a root whose own walk, which
+    // lists it, never ran: everything is resolved again)
+    const bool all = !c->walk_on || left > (n >> kWalkOffShift);
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < bs.G; g += gridDim.x * blockDim.x)
+        bs.gbest[g] = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        c->best = 0;   // (first used after a barrier, or by this block alone)
+        c->qmax = 0;
+        if (all) c->nrep = 0;
+        c->rounds_detect += 1;
+        c->items_detect += n;
+    }
+    __syncthreads();
+    // (test only: wait for one block more than exists, so the wait expires)
+    if (stall_test && !grid_barrier(c, nblocks + 1u)) return;
+    if (all || left > 0) {
+        if (!jump_resolve<RATIO>(n, F, all, max_detect, max_value, ws, bs, &s_cnt)) return;
+    }
     evaluate_tail<RATIO>(n, N2, F, ws, bs, s_key);
+}
+
+// SMs of the current device.
+static int evaluate_sms() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    return sms;
+}
+
+template <bool RATIO>
+static void launch_walk_as(int n, const Workspace &ws, const BatchState &bs, cudaStream_t st) {
+    int blocks = (n + kWalkThreads - 1) / kWalkThreads;
+    const int resident = 8 * evaluate_sms();
+    if (resident > 0 && blocks > resident) blocks = resident;
+    walk_kernel<RATIO><<<blocks, kWalkThreads, 0, st>>>(n, ws, bs);
+}
+
+static void launch_walk(int n, const Workspace &ws, const BatchState &bs, bool ratio,
+                        cudaStream_t st) {
+    if (ratio) launch_walk_as<true>(n, ws, bs, st);
+    else launch_walk_as<false>(n, ws, bs, st);
 }
 
 static int ceil_log2(long long x) {
@@ -843,13 +1155,15 @@ int launch_evaluate(int n, long long N2, Workspace ws, int stall_test, BatchStat
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     prof_begin(kProfEvaluate, st);
+    launch_walk(n, ws, bs, ratio, st);
+    const cudaError_t e0 = cudaGetLastError();
     cudaError_t e =
         ratio ? cudaLaunchKernelEx(&cfg, evaluate_kernel<true>, n, N2, max_detect, max_value,
                                    stall_test, ws, bs)
               : cudaLaunchKernelEx(&cfg, evaluate_kernel<false>, n, N2, max_detect, max_value,
                                    stall_test, ws, bs);
     prof_end(kProfEvaluate, st);
-    return e == cudaSuccess ? 1 : -1;
+    return e0 == cudaSuccess && e == cudaSuccess ? 2 : -1;
 }
 
 // --------------------------------------------------------------- extract --
@@ -1070,11 +1384,11 @@ int launch_extract(int n, int Lstar, Workspace ws, int *cycle_out, int grid, int
 }
 
 __global__ void __launch_bounds__(kThreads)
-outputs_kernel(int n, Workspace ws, int64_t *eta_num, int32_t *eta_den, int64_t *potential,
-               int32_t *policy) {
+outputs_kernel(int n, Workspace ws, BatchState bs, int64_t *eta_num, int32_t *eta_den,
+               int64_t *potential, int32_t *policy) {
     const int stride = gridDim.x * blockDim.x;
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        const JLS st = final_value(ws.jls[0], n, v);
+        const JLS st = final_value(ws.jls[bs.G ? bs.gconv[bs.gid[v]] - 1 : 0], n, v);
         int i = ws.cid_of_root[~st.J];
         if (eta_num) eta_num[v] = ws.cyc_p[i];
         if (eta_den) eta_den[v] = ws.cyc_q[i];
@@ -1083,12 +1397,12 @@ outputs_kernel(int n, Workspace ws, int64_t *eta_num, int32_t *eta_den, int64_t 
     }
 }
 
-void launch_outputs(int n, Workspace ws, int64_t *eta_num, int32_t *eta_den, int64_t *potential,
+void launch_outputs(int n, Workspace ws, BatchState bs, int64_t *eta_num, int32_t *eta_den, int64_t *potential,
                     int32_t *policy, cudaStream_t st) {
     int blocks = (n + kThreads - 1) / kThreads;
     if (blocks > 8192) blocks = 8192;
     prof_begin(kProfExtract, st);
-    outputs_kernel<<<blocks, kThreads, 0, st>>>(n, ws, eta_num, eta_den, potential, policy);
+    outputs_kernel<<<blocks, kThreads, 0, st>>>(n, ws, bs, eta_num, eta_den, potential, policy);
     prof_end(kProfExtract, st);
 }
 

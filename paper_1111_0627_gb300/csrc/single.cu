@@ -124,7 +124,7 @@ static __device__ __forceinline__ void heavy_scan(int want, int k, const int *__
 
 
 // Vertex u joins level k through edge e: its policy, its final path sums
-// (both buffers of the value jumping) and its record for the sweep, all
+// (this evaluation's value buffer), its step for the next evaluation and its record for the sweep, all
 // relative to the chosen cycle (root rstar, mean P/Q, rank RK).
 static __device__ __forceinline__ void take_edge(int u, int e, int k, int rstar, long long P,
                                                  long long Q, int RK, bool ratio, int sign,
@@ -136,17 +136,18 @@ static __device__ __forceinline__ void take_edge(int u, int e, int k, int rstar,
     ws.pi[u] = e;
     ws.succ[u] = t;
     ws.wpi[u] = wv;
-    const JLS st = ws.jls[0][t];
+    const int F = ws.ctrl->iter & 1;   // this evaluation's value buffer
+    unmark_cycle(ws, F, u);
+    const JLS st = ws.jls[F][t];
     const JLS su{~rstar, st.len + 1, st.S + (long long)wv};
-    ws.jls[0][u] = su;
-    ws.jls[1][u] = su;
+    ws.jls[F][u] = su;
+    store_step(ws, F + 1, u, t, wv);
     long long T = su.len;
     if (ratio) {
         const int tr = ws.transit[e];
         ws.tpi[u] = tr;
-        T = ws.jt[0][t] + tr;
-        ws.jt[0][u] = T;
-        ws.jt[1][u] = T;
+        T = path_time(ws.jt[F][t]) + tr;
+        ws.jt[F][u] = T;
         ws.recp[u] = P;
     }
     Rec r;
@@ -201,15 +202,16 @@ connect_kernel(const int *__restrict__ row_ptr, const int *__restrict__ col,
     const int hcap = n - H;   // a vertex that finds the list full is walked where it is met
 
     // level 0: the vertices whose policy path ends on the chosen cycle
+    const JLS *fin = ws.jls[c->iter & 1];
     int mine = 0, hmine = 0;
     for (int v = gtid; v < n; v += stride) {
-        const bool in0 = (~ws.jls[0][v].J == rstar);
+        const bool in0 = (~fin[v].J == rstar);
         sg.lev[v] = in0 ? 0 : -1;
         mine += !in0;
     }
     for (int i = gtid; i < H; i += stride) {
         pick[i] = INT_MAX;
-        hmine += ~ws.jls[0][hv[i]].J != rstar;
+        hmine += ~fin[hv[i]].J != rstar;
     }
     bool ok;
     // vertices still unconnected, heavy ones among them

@@ -111,7 +111,7 @@ void launch_check_row_ptr(const int *row_ptr, int n, int m, Ctrl *ctrl, cudaStre
 __global__ void __launch_bounds__(kSweepMaxThreads, 3)
 init_policy_kernel(const int *__restrict__ row_ptr, const int *__restrict__ col,
                    const int *__restrict__ w, int sign, int n, const int *__restrict__ gid,
-                   const int *__restrict__ init, int local_R, int count_win, int groups,
+                   const int *__restrict__ init, int local_R, int count_win, int groups, int seed,
                    Workspace ws) {
     constexpr int kWarps = kSweepMaxThreads / 32;
     __shared__ int s_maxw[kWarps];
@@ -125,8 +125,10 @@ init_policy_kernel(const int *__restrict__ row_ptr, const int *__restrict__ col,
     const int stride = gridDim.x * blockDim.x;
     const int *__restrict__ tt = ws.transit;
     int maxabs = 0, maxt = 0;
-    if (local_R)
-        for (int v = blockIdx.x * blockDim.x + tid; v < n; v += stride) ws.root_mark[v] = 0;
+    for (int v = blockIdx.x * blockDim.x + tid; v < n; v += stride) {
+        ws.root_mark[v] = 0;
+        if (seed) ws.cyc_tag[v] = 0;
+    }
     const int4 *__restrict__ grp_tab = ws.band_grp;
     const int total = grp_tab[groups].x;
     const int warps = stride >> 5;
@@ -255,8 +257,13 @@ init_policy_kernel(const int *__restrict__ row_ptr, const int *__restrict__ col,
             ws.pi[v] = be;
             ws.succ[v] = ((unsigned)t < (unsigned)n) ? t : 0;
             ws.wpi[v] = sign * (x == INT_MIN ? 0 : x);
-            if (tt) ws.tpi[v] = __ldg(&tt[be]);
-            ws.sw_iter[v] = 0;   // the first evaluation treats every vertex as changed
+            if (tt) {
+                ws.tpi[v] = __ldg(&tt[be]);
+                ws.jt[0][v] = ws.jt[1][v] = 0;   // (no tag of this solve's evaluations)
+            }
+            if (seed)   // the first evaluation's one-step state
+                ws.jls[0][v] = JLS{((unsigned)t < (unsigned)n) ? t : 0, 1,
+                                   (long long)(sign * (x == INT_MIN ? 0 : x))};
         }
     }
 #pragma unroll
@@ -580,7 +587,6 @@ improve_kernel(const int *__restrict__ row_ptr, const int *__restrict__ col,
     if (frontier != FRONTIER) return;
     __shared__ int s_sw;
     const int tid = threadIdx.x;
-    // a vertex switched here is "dirty" for the next evaluation
     const int next_eval = ws.ctrl->iter + 1;
     const int lane = tid & 31;
     if (tid == 0) s_sw = 0;
@@ -718,11 +724,12 @@ improve_kernel(const int *__restrict__ row_ptr, const int *__restrict__ col,
         // own.e == INT_MAX except in the lane that met the policy edge
         if (valid && own.e != INT_MAX) {
             if (best.rank > own.rank || (best.rank == own.rank && best.key > own.key)) {
+                const int sv = __ldg(&col[best.e]), wv = sign * __ldg(&w[best.e]);
                 ws.pi[v] = best.e;
-                ws.succ[v] = __ldg(&col[best.e]);
-                ws.wpi[v] = sign * __ldg(&w[best.e]);
+                ws.succ[v] = sv;
+                ws.wpi[v] = wv;
                 if (RATIO) ws.tpi[v] = __ldg(&ws.transit[best.e]);
-                ws.sw_iter[v] = next_eval;
+                store_step(ws, next_eval, v, sv, wv);
                 if (bs.G) {
                     const int g = bs.gid[v];
                     if (bs.gsw[g] != next_eval) bs.gsw[g] = next_eval;
@@ -845,7 +852,7 @@ heavy_init_chunk_kernel(const int *__restrict__ row_ptr, const int *__restrict__
 __global__ void __launch_bounds__(kHeavyThreads)
 heavy_init_final_kernel(const int *__restrict__ row_ptr, const int *__restrict__ col,
                         const int *__restrict__ w, int sign, int n,
-                        const int *__restrict__ init, Workspace ws) {
+                        const int *__restrict__ init, int seed, Workspace ws) {
     __shared__ Cand s_w[kHeavyThreads / 32];
     const int H = ws.ctrl->cls_cnt[kClasses];
     const int *hv = ws.cls_list + ws.ctrl->cls_off[kClasses];
@@ -869,8 +876,13 @@ heavy_init_final_kernel(const int *__restrict__ row_ptr, const int *__restrict__
             ws.pi[v] = e;
             ws.succ[v] = ((unsigned)t < (unsigned)n) ? t : 0;
             ws.wpi[v] = sign * (x == INT_MIN ? 0 : x);
-            if (ws.transit) ws.tpi[v] = __ldg(&ws.transit[e]);
-            ws.sw_iter[v] = 0;
+            if (ws.transit) {
+                ws.tpi[v] = __ldg(&ws.transit[e]);
+                ws.jt[0][v] = ws.jt[1][v] = 0;
+            }
+            if (seed)
+                ws.jls[0][v] = JLS{((unsigned)t < (unsigned)n) ? t : 0, 1,
+                                   (long long)(sign * (x == INT_MIN ? 0 : x))};
         }
     }
 }
@@ -894,7 +906,7 @@ static int init_grid() {
 
 void launch_init_policy(const int *row_ptr, const int *col, const int *w, int sign, int n, int m,
                         const int *init, Workspace ws, const BatchState *bs, cudaStream_t st,
-                        int local_R, int count_win, int band_blocks) {
+                        int local_R, int count_win, int band_blocks, int seed) {
     // one wave of co-resident blocks (the tasks are taken grid-stride)
     int blocks = (n + kSweepMaxThreads - 1) / kSweepMaxThreads;
     const int resident = init_grid();
@@ -904,7 +916,7 @@ void launch_init_policy(const int *row_ptr, const int *col, const int *w, int si
     prof_begin(kProfInit, st);
     init_policy_kernel<<<blocks, kSweepMaxThreads, 0, st>>>(row_ptr, col, w, sign, n,
                                                             bs ? bs->gid : nullptr, init, local_R,
-                                                            count_win, groups, ws);
+                                                            count_win, groups, seed, ws);
     // heavy vertices (their count is on the device: fixed grids, grid-stride)
     int cb = (m / kHeavyChunk) + 1;
     if (cb > 1024) cb = 1024;
@@ -912,7 +924,8 @@ void launch_init_policy(const int *row_ptr, const int *col, const int *w, int si
     if (fb > 1024) fb = 1024;
     heavy_init_chunk_kernel<<<cb, kHeavyThreads, 0, st>>>(row_ptr, col, w, sign, n,
                                                          bs ? bs->gid : nullptr, ws);
-    heavy_init_final_kernel<<<fb, kHeavyThreads, 0, st>>>(row_ptr, col, w, sign, n, init, ws);
+    heavy_init_final_kernel<<<fb, kHeavyThreads, 0, st>>>(row_ptr, col, w, sign, n, init, seed,
+                                                         ws);
     prof_end(kProfInit, st);
 }
 
@@ -1024,11 +1037,12 @@ improve_heavy_final_kernel(const int *__restrict__ col, const int *__restrict__ 
             long long cur_key = (long long)r.w * (long long)ws.wpi[v] + V;
             if (RATIO) cur_key -= __ldg(&ws.recp[t]) * (long long)ws.tpi[v];
             if (best.rank > r.z || (best.rank == r.z && best.key > cur_key)) {
+                const int sv = __ldg(&col[best.e]), wv = sign * __ldg(&w[best.e]);
                 ws.pi[v] = best.e;
-                ws.succ[v] = __ldg(&col[best.e]);
-                ws.wpi[v] = sign * __ldg(&w[best.e]);
+                ws.succ[v] = sv;
+                ws.wpi[v] = wv;
                 if (RATIO) ws.tpi[v] = __ldg(&ws.transit[best.e]);
-                ws.sw_iter[v] = next_eval;
+                store_step(ws, next_eval, v, sv, wv);
                 if (bs.G) {
                     const int g = bs.gid[v];
                     if (bs.gsw[g] != next_eval) bs.gsw[g] = next_eval;

@@ -58,9 +58,10 @@ static __device__ __forceinline__ int decide(int v, const Cand &b, const CurKey 
     }
     if (!(b.rank > c.rank || (b.rank == c.rank && b.key > c.key))) return 0;
     ws.pi[v] = b.e;
-    ws.succ[v] = colp[b.e - base];
-    ws.wpi[v] = sign * wp[b.e - base];
-    ws.sw_iter[v] = next_eval;
+    const int sv = colp[b.e - base], wv = sign * wp[b.e - base];
+    ws.succ[v] = sv;
+    ws.wpi[v] = wv;
+    store_step(ws, next_eval, v, sv, wv);
     if (bs.G) {
         const int g = bs.gid[v];
         if (bs.gsw[g] != next_eval) bs.gsw[g] = next_eval;

@@ -295,9 +295,10 @@ improve_window_kernel(const int *__restrict__ row_ptr, const int *__restrict__ c
             if (valid && own.e != INT_MAX &&
                 (best.rank > own.rank || (best.rank == own.rank && best.key > own.key))) {
                 ws.pi[v] = best.e;
-                ws.succ[v] = __ldg(&col[best.e]);
-                ws.wpi[v] = sign * __ldg(&w[best.e]);
-                ws.sw_iter[v] = next_eval;
+                const int sv = __ldg(&col[best.e]), wv = sign * __ldg(&w[best.e]);
+                ws.succ[v] = sv;
+                ws.wpi[v] = wv;
+                store_step(ws, next_eval, v, sv, wv);
                 if (bs.G) {
                     const int gg = bs.gid[v];
                     if (bs.gsw[gg] != next_eval) bs.gsw[gg] = next_eval;
