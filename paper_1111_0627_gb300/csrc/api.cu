@@ -235,7 +235,7 @@ static int persistent_grid() {
 static int map_err_bits(int err) {
     if (err & kErrTimeout) return OCM_ERR_TIMEOUT;
     if (err & (kErrInitPolicy | kErrTransit | kErrUnreached)) return OCM_ERR_INVALID_ARG;
-    if (err & kErrRatioKey) return OCM_ERR_OVERFLOW;
+    if (err & (kErrRatioKey | kErrRange)) return OCM_ERR_OVERFLOW;
     if (err & (kErrRowPtr | kErrCol)) return OCM_ERR_BAD_CSR;
     if (err & kErrNoOutEdge) return OCM_ERR_NO_OUT_EDGE;
     if (err & kErrWeightMin) return OCM_ERR_OVERFLOW;
@@ -631,6 +631,9 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
     auto phase = [](const char *name) { nvtxRangePop(); nvtxRangePushA(name); };
     nvtxRangePushA("ocm:validate");
     struct PopOnExit { ~PopOnExit() { nvtxRangePop(); } } pop_phase;
+    const int req_kind = opt ? opt->sweep_kind : OCM_SWEEP_DEFAULT;
+    const bool outputs =
+        opt && (opt->eta_num || opt->eta_den || opt->potential || opt->policy);
     // the frontier sweep: not in the single-lambda form, whose rebuild writes
     // records after the record pass
     const int frontier =
@@ -656,7 +659,6 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
     // (the edge-tiled sweep has no cycle-ratio form)
     // (the window sweep is decided after the initial pass, which measures the
     // locality it relies on; it groups vertices by the same degree classes)
-    const int req_kind = opt ? opt->sweep_kind : OCM_SWEEP_DEFAULT;
     int kind = (req_kind == OCM_SWEEP_TILES && !ratio) ? OCM_SWEEP_TILES : OCM_SWEEP_CLASSES;
     int epl = (opt && opt->edges_per_lane > 0) ? opt->edges_per_lane : kEdgesPerLane;
     if (epl > 64) epl = 64;
@@ -733,10 +735,9 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
     //     serves for every graph.
     if (bs) {
         const int small_n = opt ? opt->batch_small_vertices : 0;   // 0: automatic
-        const bool outputs = opt && (opt->eta_num || opt->eta_den || opt->potential || opt->policy);
         if (small_n >= 0 && !ratio && !outputs) {
-            const int k = launch_batch_small(row_ptr, col_idx, w, sign, small_n, n, max_iters,
-                                             b.small_queue, ws, b, st);
+            const int k = launch_batch_small(row_ptr, col_idx, w, sign, small_n, n, h.max_ng, max_iters,
+                                             opt && opt->init_policy ? 1 : 0, b.small_queue, ws, b, st);
             if (k < 0) return OCM_ERR_CUDA;
             launches += k;
         }
@@ -833,7 +834,7 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
         }
         launches += launch_extract(n, Lstar, ws, out.cycle_out, grid, local_R, st);
     }
-    if (opt && (opt->eta_num || opt->eta_den || opt->potential || opt->policy)) {
+    if (outputs) {
         launch_outputs(n, ws, b, opt->eta_num, opt->eta_den, opt->potential, opt->policy, st);
         launches += 1;
     }

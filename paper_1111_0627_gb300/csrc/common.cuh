@@ -143,7 +143,9 @@ struct Ctrl {
     int small_bucket[32];     // graphs per size bucket floor(log2 n_g)
     int small_cursor[32];     // fill cursors of the buckets
     int small_total;          // graphs in the queue
-    int small_head;           // next queue position to pop
+    int small_big;            // the first of them, solved by a cluster each
+    int small_head;           // next queue position to pop, counted from small_big
+    int big_head;             // the same among the first small_big
     int small_iters;          // largest iteration count among them
     int node_cnt;             // two-level evaluation: exits listed (nodes of the contracted graph)
     int fix_k;                // two-level evaluation: roots found on the node graph (capped)
@@ -171,6 +173,7 @@ struct Ctrl {
     int old_roots;            // roots listed and settled before the walks
     int jump_rounds;
     int walk_fail;            // walks were dropped before in this solve
+    int team_off;             // a solve by one team met a vertex of more than kHeavyEdges edges
 };
 
 // One-level evaluation: walks that leave more than n >> kWalkOffShift
@@ -220,6 +223,7 @@ enum : int {
     kErrTransit = 1024,   // a transit time below 1
     kErrRatioKey = 2048,  // cycle ratio: the exact order keys of the current cycles overflow int64
     kErrUnreached = 4096, // single-lambda rebuild: a vertex cannot reach the chosen cycle
+    kErrRange = 16384,    // the exactness bound of the weights (solve by one team)
     kErrConnect = 8192,   // single-lambda rebuild: inconsistent state (no chosen cycle, no edge)
 };
 
@@ -455,6 +459,15 @@ __device__ __forceinline__ int warp_append(int *counter, bool pred, int lane) {
 __device__ __forceinline__ long long gcd_ll(long long a, long long b) {
     if (a < 0) a = -a;
     if (b < 0) b = -b;
+    if (((a | b) >> 32) == 0) {   // (a 64-bit remainder takes several times a 32-bit one)
+        unsigned x = (unsigned)a, y = (unsigned)b;
+        while (y != 0) {
+            const unsigned t = x % y;
+            x = y;
+            y = t;
+        }
+        return (long long)x;
+    }
     while (b != 0) {
         long long t = a % b;
         a = b;
@@ -527,8 +540,8 @@ int prepare_evaluate_local();
 int evaluate_local_blocks(int n);
 int launch_batch_prepare(int N, int M, BatchState bs, Workspace ws, cudaStream_t st);
 int launch_batch_small(const int *row_ptr, const int *col, const int *w, int sign, int max_n,
-                       long long N, long long max_iters, int *queue, Workspace ws, BatchState bs,
-                       cudaStream_t st);
+                       long long N, int max_ng, long long max_iters, int warm, int *queue,
+                       Workspace ws, BatchState bs, cudaStream_t st);
 int launch_batch_finish(int N, int sign, int Lbits, BatchState bs, Workspace ws, int64_t *num,
                         int32_t *den, int32_t *cycle_len, int32_t *cycle_out, int grid,
                         cudaStream_t st);
