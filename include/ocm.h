@@ -270,7 +270,8 @@ typedef struct ocm_stats {
     int64_t launches;       /* kernels launched by this call                        */
     int64_t detect_items;   /* vertices evaluated, summed over iterations           */
     int64_t value_items;    /* 0                                                    */
-    int32_t graph_loop;     /* 1: the iteration ran as a CUDA graph, 0: host-driven */
+    int32_t graph_loop;     /* 1: the iteration ran on the device (a CUDA graph, or the
+                           one launch of a small solve), 0: host-driven */
     int32_t rebuild_levels; /* OCM_FLAG_SINGLE_LAMBDA: backward-search levels of the
                                rebuilds, summed over iterations; 0 otherwise         */
     int32_t batch_small_graphs; /* ocm_solve_batch: graphs solved one per thread block

@@ -19,7 +19,7 @@ CSRC = os.path.join(_PKG, "csrc")
 BUILD = os.path.join(_PKG, "_build")
 LIB_PATH = os.path.join(BUILD, "libocm.so")
 INCLUDE = os.path.join(_ROOT, "include")
-SOURCES = ["sweep.cu", "sweep_tiles.cu", "sweep_window.cu", "evaluate.cu", "batch.cu", "batch_small.cu", 
+SOURCES = ["sweep.cu", "sweep_tiles.cu", "sweep_window.cu", "evaluate.cu", "batch.cu", "batch_small.cu", "solve_team.cu",
            "api.cu", "static_ws.cu", "scc.cu", "single.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",

@@ -634,6 +634,46 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
     const int req_kind = opt ? opt->sweep_kind : OCM_SWEEP_DEFAULT;
     const bool outputs =
         opt && (opt->eta_num || opt->eta_den || opt->potential || opt->policy);
+    // A small graph with no form asked for: the whole solve by one block or
+    // cluster.  (A host-driven or profiled loop, and the fallback to one, keep
+    // the launch per step.)
+    if (!bs && !ratio && (!opt || (opt->flags == 0 && opt->edges_per_lane <= 0 &&
+                                   opt->sweep_threads <= 0 && req_kind == OCM_SWEEP_DEFAULT)) &&
+        team_solves(n, m) && !prof_active() && !injected_fault("alloc")) {
+        const long long cap = (opt && opt->max_iters > 0) ? opt->max_iters : 4LL * n + 64;
+        const int k = launch_solve_team(row_ptr, col_idx, w, sign, n, m,
+                                        opt ? opt->init_policy : nullptr, cap, out.cycle_out, ws, st);
+        if (k < 0) return OCM_ERR_CUDA;
+        launches += k;
+        int rc = read_ctrl(ws.ctrl, &h, st);
+        if (rc) return rc;
+        if (h.err) return map_err_bits(h.err);
+        if (!h.team_off) {   // (else a hub, which the general path spreads over the grid)
+            if (h.not_converged) return OCM_ERR_NOT_CONVERGED;
+            if (h.res_len < 1 || h.cnt[0] != h.res_len) return OCM_ERR_INTERNAL;
+            if (outputs) {
+                launch_outputs(n, ws, b, opt->eta_num, opt->eta_den, opt->potential, opt->policy, st);
+                launches += 1;
+                if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
+                    return OCM_ERR_CUDA;
+            }
+            *out.num = (int64_t)sign * (int64_t)h.res_num;
+            *out.den = h.res_den;
+            *out.cycle_len = h.res_len;
+            if (stats) {
+                memset(stats, 0, sizeof *stats);
+                stats->iterations = h.iter;
+                stats->cycles = h.res_cycles;
+                stats->detect_rounds = h.rounds_detect;
+                stats->switched = h.switched_total;
+                stats->launches = launches;
+                stats->detect_items = h.items_detect;
+                stats->graph_loop = 1;
+                stats->sweep_kind = OCM_SWEEP_CLASSES;
+            }
+            return OCM_OK;
+        }
+    }
     // the frontier sweep: not in the single-lambda form, whose rebuild writes
     // records after the record pass
     const int frontier =

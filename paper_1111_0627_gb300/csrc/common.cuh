@@ -542,6 +542,11 @@ int launch_batch_prepare(int N, int M, BatchState bs, Workspace ws, cudaStream_t
 int launch_batch_small(const int *row_ptr, const int *col, const int *w, int sign, int max_n,
                        long long N, int max_ng, long long max_iters, int warm, int *queue,
                        Workspace ws, BatchState bs, cudaStream_t st);
+// Whole solve of a small graph in one launch (solve_team.cu).
+bool team_solves(int n, int m);
+int launch_solve_team(const int *row_ptr, const int *col, const int *w, int sign, int n, int m,
+                      const int *init, long long max_iters, int *cycle_out, Workspace ws,
+                      cudaStream_t st);
 int launch_batch_finish(int N, int sign, int Lbits, BatchState bs, Workspace ws, int64_t *num,
                         int32_t *den, int32_t *cycle_len, int32_t *cycle_out, int grid,
                         cudaStream_t st);
