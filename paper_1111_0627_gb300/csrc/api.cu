@@ -258,72 +258,6 @@ static int read_ctrl(const Ctrl *dev, Ctrl *host, cudaStream_t st) {
 // the control block, so the same launches serve a host-driven loop and the
 // body of a CUDA graph WHILE node.
 
-// Ends a step: stop on an error or when no vertex switched (Howard's
-// termination test, Alg. 1), else advance the iteration index unless the
-// cap is reached.  With use_cond the decision also sets the WHILE node's
-// condition.
-// It also prepares the counters the next evaluation starts from, and decides
-// whether its record pass marks the records it changes (frontier sweep).
-// One warp: the one-level evaluation's marked cycles that no switch broke stay
-// listed, and their roots are settled for the next evaluation.
-__global__ void loop_control_kernel(Workspace ws, BatchState bs, int n, long long max_iters, int use_cond,
-                                    cudaGraphConditionalHandle handle) {
-    Ctrl *c = ws.ctrl;
-    int kept = 0;
-    const bool more = c->err == 0 && c->changed && (long long)c->iter + 1 < max_iters;
-    if (more && ws.walk && c->nrep <= kSettleRoots) {
-        JLS *next = ws.jls[(c->iter + 1) & 1];
-        const int tag = c->iter + 2;   // of the next evaluation
-        const int lane = threadIdx.x;
-        for (int base = 0; base < c->nrep; base += 32) {
-            const int r = base + lane < c->nrep ? ws.cyc_root[base + lane] : -1;
-            const bool keep =
-                r >= 0 && (ws.root_mark[r] & 1) && !(bs.G && bs.gconv[bs.gid[r]]);
-            const unsigned m = __ballot_sync(0xffffffffu, keep);
-            if (keep) {
-                const int pos = kept + __popc(m & ((1u << lane) - 1u));   // (<= base + lane)
-                ws.cyc_root[pos] = r;
-                ws.cid_of_root[r] = pos;
-                ws.root_mark[r] = (tag << 1) | 1;
-                next[r] = JLS{~r, 0, 0};
-            }
-            kept += __popc(m);
-            __syncwarp();
-        }
-    }
-    __syncwarp();
-    if (threadIdx.x) return;
-    // the next step's cooperative launches count their barriers from zero
-    for (int i = 0; i < 2; ++i) {
-        c->bar[i].arrive = 0;
-        for (int j = 0; j < 4; ++j) {
-            c->bar[i].sum[j] = 0;
-            c->bar[i].sum2[j] = 0;
-        }
-    }
-    c->switched_total += c->switched;
-    if (more) c->iter += 1;
-    else if (c->err == 0 && c->changed) c->not_converged = 1;
-    c->mark = c->frontier == 2 ||
-              (c->frontier && (long long)c->switched < ((long long)n >> kFrontierSwitchShift));
-    c->dirty_on = c->mark;
-    c->dirty_cnt = 0;
-    c->changed = 0;
-    c->switched = 0;
-    if (more) {
-        c->nrep = kept;
-        c->old_roots = kept;
-    }
-    if (c->walk_on && c->walk_left > (n >> kWalkOffShift)) {
-        c->walk_on = 0;
-        c->walk_fail = 1;
-    }
-    if (!c->walk_on) c->walk_on = !c->walk_fail || c->jump_rounds <= kWalkRounds;
-    c->walk_left = 0;
-    c->loop_more = more ? 1 : 0;
-    if (use_cond) cudaGraphSetConditional(handle, more ? 1u : 0u);
-}
-
 // Everything a step's launches depend on.
 struct StepArgs {
     const int32_t *row_ptr, *col_idx, *w;
@@ -363,7 +297,7 @@ static int launch_step(const StepArgs &a, int use_cond, cudaGraphConditionalHand
     if (ks < 0) return -1;
     int k = le + ks;
     if (a.batch) k += launch_batch_converge(a.bs, a.ws, st);
-    loop_control_kernel<<<1, 32, 0, st>>>(a.ws, a.bs, a.n, a.max_iters, use_cond, handle);
+    launch_loop_control(a.n, a.max_iters, a.ws, a.bs, use_cond, handle, st);
     k += 1;
     if (cudaGetLastError() != cudaSuccess) return -1;
     return k;

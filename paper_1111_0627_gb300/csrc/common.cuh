@@ -173,6 +173,9 @@ struct Ctrl {
     int old_roots;            // roots listed and settled before the walks
     int jump_rounds;
     int walk_fail;            // walks were dropped before in this solve
+    int walk_deep;            // the next walks publish their parts (deep policies, evaluate.cu)
+    unsigned long long depth_sum;   // path lengths of the policy just evaluated, of every eighth
+    int depth_cnt;                  // block's vertices: their sum, and how many
     int team_off;             // a solve by one team met a vertex of more than kHeavyEdges edges
 };
 
@@ -183,8 +186,13 @@ struct Ctrl {
 // walks if it is at most kWalkRounds.  The first evaluation of a cold start
 // jumps: the heaviest edges form a random mapping, about sqrt(n) deep.
 constexpr int kWalkOffShift = 3;
+// Deep policies (an average path of more than kWalkDeep steps) walk with
+// published parts, up to kWalkDeepRounds.
 constexpr int kWalkSteps = 256;
 constexpr int kWalkRounds = 9;
+constexpr int kWalkDeep = 48;
+constexpr int kWalkDeepRounds = 12;
+constexpr int kWalkDeepGraphs = 64;  // (of a batch: active graphs at most)
 constexpr int kSettleRoots = 1024;   // roots settled ahead of the walks at most
 
 // The record pass marks the records it changes when the sweep before it
@@ -534,6 +542,8 @@ int launch_sweep_tiles(const int *row_ptr, const int *col, const int *w, int sig
 int launch_batch_converge(BatchState bs, Workspace ws, cudaStream_t st);
 int launch_classify(const int *row_ptr, int n, int epl, int band_blocks, Workspace ws,
                     cudaStream_t st);
+void launch_loop_control(int n, long long max_iters, Workspace ws, BatchState bs, int use_cond,
+                         cudaGraphConditionalHandle handle, cudaStream_t st);
 int launch_evaluate(int n, long long N2, Workspace ws, int stall_test, BatchState bs,
                     cudaStream_t st, bool local = false, bool no_bitmap = false);
 int prepare_evaluate_local();

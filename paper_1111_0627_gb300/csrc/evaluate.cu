@@ -402,6 +402,9 @@ static __device__ void evaluate_tail(int n, long long N2, int F, const Workspace
     // word of the change bitmap, in each of its kMU slots; the slots' loads
     // are issued together, stage by stage)
     constexpr int kMU = 4;
+    const bool tally = !ratio && !LOCAL && (blockIdx.x & 7) == 0;
+    long long depth = 0;   // (path lengths, for the choice of the next walks)
+    int resolved = 0;
     int changed = 0;
     for (int base0 = first + (int)threadIdx.x - lane; base0 < n; base0 += kMU * stride) {
         JLS st[kMU];
@@ -443,6 +446,10 @@ static __device__ void evaluate_tail(int n, long long N2, int F, const Workspace
                 const int q = tab_q[i];
                 Rec rec;
                 const long long T = ratio ? path_time(ws.jt[F][v]) : (long long)st[u].len;
+                if (tally) {
+                    depth += st[u].len;
+                    ++resolved;
+                }
                 rec.V = (long long)q * st[u].S - p * T;
                 rec.rank = tab_rank[i];
                 rec.q = q;
@@ -468,6 +475,27 @@ static __device__ void evaluate_tail(int n, long long N2, int F, const Workspace
                     }
                 }
             }
+        }
+    }
+    if (tally) {
+        __shared__ unsigned long long s_depth;
+        __shared__ int s_resolved;
+        if (threadIdx.x == 0) {
+            s_depth = 0;
+            s_resolved = 0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) depth += __shfl_xor_sync(0xffffffffu, depth, o);
+        resolved = __reduce_add_sync(0xffffffffu, resolved);
+        if (lane == 0 && resolved) {
+            atomicAdd(&s_depth, (unsigned long long)depth);
+            atomicAdd(&s_resolved, resolved);
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && s_resolved) {
+            atomicAdd(&c->depth_sum, s_depth);
+            atomicAdd(&c->depth_cnt, s_resolved);
         }
     }
     if (mark) {
@@ -526,10 +554,23 @@ static __device__ void evaluate_tail(int n, long long N2, int F, const Workspace
 //   passing the root: a walk that passed a new root before it was settled, and
 // met a settled vertex of the cycle after that, has gone round once too often;
 // walks that end at a new root look for its first occurrence.
-//   limit: a warp gives up after kWalkSteps steps or a few new cycles;
-// evaluate_kernel resolves what is left by jump rounds.  While the policy
-// graph is deep (a random first policy has paths of about sqrt(n) steps) the
-// walks are left out altogether: see kWalkRounds.
+//   samples: where no old root is left every vertex leads to a new cycle, passes
+// its root and adds its steps up again, as long as the walk itself.  There 512
+// vertices spread over the graph walk first, at the end of the step before
+// (loop_control_kernel), and settle the roots they find, so that the walks
+// start with old roots after all.
+//   deep policies (more than kWalkDeep = 48 steps on average, by the last
+// evaluation; not for the ratio, whose times do not fit the state): a walk that
+// is open after kWalkPart steps publishes the part it has walked in its own
+// state, and whoever comes by takes it in one step, so that a path of hundreds of
+// steps takes a few dozen reads.  Then nobody looks for cycles (a published part
+// could go round one without stopping at its root): what leads to a cycle that
+// is neither old nor met by a sample stays open, and is left to the jump rounds,
+// which start from the policy edges.
+//   limit: a warp gives up after kWalkSteps steps (published parts: after
+// kWalkDeepSteps) or a few new cycles; evaluate_kernel resolves what is left by
+// jump rounds.  A first policy (random: paths of about sqrt(n) steps, no old
+// root) is left to them altogether: see kWalkRounds.
 //   buffers: evaluation k reads and settles jls[k & 1], where every vertex
 // holds its one step {succ, 1, weight} at the start; a walk writes its own
 // step into the other buffer for evaluation k + 1, where the sweep's switches
@@ -543,12 +584,25 @@ static __device__ void evaluate_tail(int n, long long N2, int F, const Workspace
 // with a settled root: 54 us at n = 2.1 M (product graph), 45-50 us at n =
 // 2^20 (random graph), about twice that where a new cycle has to be found.
 // An evaluation (this kernel and the next) against the jump rounds alone,
-// averaged over a solve: 108 against 204 us and 92 against 158 us.  Reading
+// averaged over a solve: 108 against 204 us and 92 against 158 us.  A policy
+// 100 to 135 steps deep at n = 2^20: 160 us a walk without published parts, 48
+// with; 200 to 400 steps deep at n = 2.4 M (a random digraph's giant component):
+// walks failed after 2.1 ms and an evaluation took 600 us of jump rounds, 125 with.
+// Publishing from 24 steps on gained the random graphs another 4% and cost the
+// product graphs up to 8%, whose small new cycles are then left to the jump
+// rounds; a limit of 64 steps left too much open (13.7 -> 9.1 ms a solve with 128,
+// 12 ms with 64), and reading past L1 after 16 or 32 steps, to see newer parts,
+// took 10-25% longer.  Reading
 // the states past L1 took 220-360 us, and giving each lane its next vertex as
 // soon as it was done (more divergence) 100-300 us.
 // ---------------------------------------------------------------------------
 constexpr int kWalkThreads = 256;
-constexpr int kWalkTight = 32;    // steps between two looks for a cycle
+constexpr int kWalkTight = 32;    // steps up to the first look for a cycle
+constexpr int kWalkPart = 8;      // deep policies: steps between two published parts,
+constexpr int kWalkDeepSteps = 128;         // and of a walk at most
+constexpr int kWalkPublish = 1 << 23;       // longest published part (times those: an int)
+constexpr int kSampleThreads = 512;         // samples that look for cycles
+constexpr int kSampleSteps = 512;
 constexpr int kWalkCycles = 8;    // new cycles a warp looks for
 
 static __device__ __forceinline__ JLS load_state(const JLS *p) {   // (through L1)
@@ -566,10 +620,10 @@ static __device__ __forceinline__ void store_state(JLS *p, const JLS &s) {
 
 // Looks for a cycle on the path from cur.  Returns its smallest vertex, now
 // settled and listed, or -1 if the path meets a settled vertex or is too long.
-static __device__ __forceinline__ int walk_find_cycle(int cur, JLS *st, unsigned tag,
-                                                   const Workspace &ws) {
+static __device__ __forceinline__ int walk_find_cycle(int cur, JLS *st, unsigned tag, int limit,
+                                                      const Workspace &ws, int *listed) {
     int tort = cur, lam = 0, power = 1, r = -1;
-    for (int k = 0; k < 2 * kWalkSteps; ++k) {
+    for (int k = 0; k < limit; ++k) {
         const JLS s = load_state(&st[cur]);
         if (s.J < 0) return -1;
         cur = s.J;
@@ -585,7 +639,8 @@ static __device__ __forceinline__ int walk_find_cycle(int cur, JLS *st, unsigned
     }
     if (r < 0) return -1;
     int k = 0;
-    for (int y = ws.succ[cur]; y != cur && k < 2 * kWalkSteps; y = ws.succ[y], ++k) r = min(r, y);
+    for (int y = ws.succ[cur]; y != cur && k < limit; y = ws.succ[y], ++k) r = min(r, y);
+    if (k >= limit) return -1;
     store_state(&st[r], JLS{~r, 0, 0});
     // the first to find it lists the root and marks the cycle
     volatile int *mark = &ws.root_mark[r];
@@ -594,12 +649,13 @@ static __device__ __forceinline__ int walk_find_cycle(int cur, JLS *st, unsigned
         const int pos = atomicAdd(&ws.ctrl->nrep, 1);
         ws.cyc_root[pos] = r;
         ws.cid_of_root[r] = pos;
+        if (listed) atomicAdd(listed, 1);
         k = 0;
         int y = r;
         do {
             ws.cyc_tag[y] = (int)tag;
             y = ws.succ[y];
-        } while (y != r && ++k < 2 * kWalkSteps);
+        } while (y != r && ++k < limit);
         if (y == r) *mark = (int)(tag << 1) | 1;
     }
     return r;
@@ -619,6 +675,13 @@ walk_kernel(int n, Workspace ws, BatchState bs) {
     const int F = c->iter & 1;
     const unsigned tag = (unsigned)c->iter + 1u;
     const int old_roots = c->old_roots;
+    const bool deep = !RATIO && c->walk_deep;
+    if (deep && old_roots == 0) {   // (the samples found no cycle)
+        if (first + threadIdx.x == 0) c->walk_left = n;
+        return;
+    }
+    const int part = deep ? kWalkPart : kWalkTight;
+    const int steps = deep ? kWalkDeepSteps : kWalkSteps;
     JLS *st = ws.jls[F], *next = ws.jls[F ^ 1];
     const int lane = threadIdx.x & 31;
     // settled before the walks (the first entries of the root list; a new
@@ -642,10 +705,10 @@ walk_kernel(int n, Workspace ws, BatchState bs) {
         unsigned open;           // lanes still walking
         for (;;) {
 #pragma unroll 1
-            for (int k = 0; k < kWalkTight && __any_sync(0xffffffffu, s.J >= 0); ++k) {
+            for (int k = 0; k < part && __any_sync(0xffffffffu, s.J >= 0); ++k) {
                 if (s.J >= 0) {
                     if (RATIO) T += (unsigned)ws.tpi[cur];
-                    ++len;
+                    len += s.len;   // (1 unless published)
                     S += s.S;
                     cur = s.J;
                     s = load_state(&st[cur]);
@@ -660,11 +723,16 @@ walk_kernel(int n, Workspace ws, BatchState bs) {
             }
             open = __ballot_sync(0xffffffffu, s.J >= 0);
             if (!open) break;
-            total += kWalkTight;
-            if (total > kWalkSteps) break;
+            total += part;
+            if (total >= steps) break;
+            if (deep) {
+                if (s.J >= 0 && len <= kWalkPublish) store_state(&st[v], JLS{cur, len, S});
+                continue;
+            }
+            if (total & (total - 1)) continue;   // (looks after 32, 64 and 128 steps)
             const int leader = __ffs(open) - 1;
             int r = -1;
-            if (lane == leader) r = walk_find_cycle(cur, st, tag, ws);
+            if (lane == leader) r = walk_find_cycle(cur, st, tag, 2 * total, ws, nullptr);
             r = __shfl_sync(0xffffffffu, r, leader);
             if (r >= 0) {
                 if (++found > kWalkCycles) break;
@@ -708,6 +776,99 @@ walk_kernel(int n, Workspace ws, BatchState bs) {
             if (sofar > (n >> kWalkOffShift)) return;   // (evaluate_kernel resolves everything)
         }
     }
+}
+
+// Ends a step: stop on an error or when no vertex switched (Howard's
+// termination test, Alg. 1), else advance the iteration index unless the
+// cap is reached.  With use_cond the decision also sets the WHILE node's
+// condition.
+// It also prepares the counters the next evaluation starts from, and decides
+// whether its record pass marks the records it changes (frontier sweep) and
+// how it walks.
+// The first warp: the one-level evaluation's marked cycles that no switch broke
+// stay listed, and their roots are settled for the next evaluation.  The whole
+// block, where none stayed: the samples look for the new cycles.
+__global__ void __launch_bounds__(kSampleThreads)
+loop_control_kernel(Workspace ws, BatchState bs, int n, long long max_iters, int use_cond,
+                    cudaGraphConditionalHandle handle) {
+    __shared__ int s_sample;
+    Ctrl *c = ws.ctrl;
+    if (threadIdx.x < 32) {
+        int kept = 0;
+        const bool more = c->err == 0 && c->changed && (long long)c->iter + 1 < max_iters;
+        if (more && ws.walk && c->nrep <= kSettleRoots) {
+            JLS *next = ws.jls[(c->iter + 1) & 1];
+            const int tag = c->iter + 2;   // of the next evaluation
+            const int lane = threadIdx.x;
+            for (int base = 0; base < c->nrep; base += 32) {
+                const int r = base + lane < c->nrep ? ws.cyc_root[base + lane] : -1;
+                const bool keep =
+                    r >= 0 && (ws.root_mark[r] & 1) && !(bs.G && bs.gconv[bs.gid[r]]);
+                const unsigned m = __ballot_sync(0xffffffffu, keep);
+                if (keep) {
+                    const int pos = kept + __popc(m & ((1u << lane) - 1u));   // (<= base + lane)
+                    ws.cyc_root[pos] = r;
+                    ws.cid_of_root[r] = pos;
+                    ws.root_mark[r] = (tag << 1) | 1;
+                    next[r] = JLS{~r, 0, 0};
+                }
+                kept += __popc(m);
+                __syncwarp();
+            }
+        }
+        __syncwarp();
+        if (threadIdx.x == 0) {
+            // the next step's cooperative launches count their barriers from zero
+            for (int i = 0; i < 2; ++i) {
+                c->bar[i].arrive = 0;
+                for (int j = 0; j < 4; ++j) {
+                    c->bar[i].sum[j] = 0;
+                    c->bar[i].sum2[j] = 0;
+                }
+            }
+            c->switched_total += c->switched;
+            if (more) c->iter += 1;
+            else if (c->err == 0 && c->changed) c->not_converged = 1;
+            c->mark = c->frontier == 2 ||
+                      (c->frontier &&
+                       (long long)c->switched < ((long long)n >> kFrontierSwitchShift));
+            c->dirty_on = c->mark;
+            c->dirty_cnt = 0;
+            c->changed = 0;
+            c->switched = 0;
+            if (more) {
+                c->nrep = kept;
+                c->old_roots = kept;
+            }
+            // (the ratio's sums stay 0)
+            c->walk_deep = c->depth_sum > (unsigned long long)kWalkDeep * (unsigned)c->depth_cnt &&
+                           (bs.G == 0 || c->active_graphs <= kWalkDeepGraphs);
+            c->depth_sum = 0;
+            c->depth_cnt = 0;
+            if (c->walk_on && c->walk_left > (n >> kWalkOffShift)) {
+                c->walk_on = 0;
+                c->walk_fail = 1;
+            }
+            if (!c->walk_on)
+                c->walk_on = !c->walk_fail ||
+                             c->jump_rounds <= (c->walk_deep ? kWalkDeepRounds : kWalkRounds);
+            c->walk_left = 0;
+            c->loop_more = more ? 1 : 0;
+            s_sample = more && ws.walk && c->walk_on && kept == 0;
+            if (use_cond) cudaGraphSetConditional(handle, more ? 1u : 0u);
+        }
+    }
+    __syncthreads();
+    if (!s_sample) return;
+    const int v = (int)((long long)threadIdx.x * n / kSampleThreads);
+    if (bs.G && bs.gconv[bs.gid[v]]) return;
+    walk_find_cycle(v, ws.jls[c->iter & 1], (unsigned)c->iter + 1u, kSampleSteps, ws,
+                    &c->old_roots);
+}
+
+void launch_loop_control(int n, long long max_iters, Workspace ws, BatchState bs, int use_cond,
+                         cudaGraphConditionalHandle handle, cudaStream_t st) {
+    loop_control_kernel<<<1, kSampleThreads, 0, st>>>(ws, bs, n, max_iters, use_cond, handle);
 }
 
 // The first evaluation's one-step states (when the initial pass left them out).
