@@ -320,6 +320,7 @@ static __device__ __forceinline__ int team_walk(Team<C> &tm, const TeamGraph &g)
                     // nothing is settled by it before the root is, here)
                     for (y = ws.succ[r]; y != r; y = ws.succ[y])
                         team_store<SM>(&st[y], JLS{ws.succ[y], 1, (long long)ws.wpi[y]});
+                    __threadfence();   // (before anything that follows from the root)
                     team_store<SM>(&st[r], JLS{~r, 0, 0});
                 }
             }
@@ -349,6 +350,7 @@ static __device__ __forceinline__ int team_walk(Team<C> &tm, const TeamGraph &g)
                     ++k;
                 }
                 if (y == root) f = JLS{~root, k, Sy};
+                __threadfence();   // (after the cycle's states were put back, above)
             }
             team_store<SM>(&st[v], f);
         }
