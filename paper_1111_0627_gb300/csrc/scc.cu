@@ -37,10 +37,17 @@ constexpr int kSccThreads = 1024;   // one block per SM: fewer arrivals at each 
 constexpr int kSortThreads = 512;
 constexpr int kScanBlock = 1024;
 constexpr int kTrimRounds = 8;
-constexpr int kActive = 1, kFw = 2, kBw = 4;
+constexpr int kTrimU = 4;           // vertices per thread per pass of a trimming round
+constexpr unsigned long long kActive = 1, kFw = 2, kBw = 4, kReached = kFw | kBw;
 // A frontier vertex with more edges than this in the search direction goes to
 // a heavy frontier, whose vertices are expanded by the whole grid together.
 constexpr int kSccHeavy = 2048;
+
+// State of an active vertex of a class that no search has reached.
+static __host__ __device__ __forceinline__ unsigned long long scc_key(int color) {
+    return ((unsigned long long)color << 3) | kActive;
+}
+static __device__ __forceinline__ int scc_color(unsigned long long st) { return (int)(st >> 3); }
 
 // Workspace of the decomposition, carved from one caller buffer.
 struct SccWs {
@@ -48,8 +55,9 @@ struct SccWs {
     int *in_src;     // [m] source vertex of each in-edge
     int *cursor;     // [n] CSC scatter cursors
     int *bsum;       // [n / kScanBlock + 1] block sums of the scans
-    int *color;      // [n] colour class (3p + k after a split at pivot p; 3n at first)
-    int *flags;      // [n] kActive | kFw | kBw
+    unsigned long long *state;   // [n] colour class (3p + k after a split at pivot p; 3n at
+                     //   first) * 8 + kActive | kFw | kBw; 0 once the component is known
+                     //   (one word: the random reads of a neighbour take one sector, not two)
     int *piv;        // [3n + 1] pivot of each class
     int *minv;       // [n] smallest vertex of the component found from pivot p
     int *q[4];       // [n] BFS frontiers: forward 0/1, backward 2/3
@@ -74,8 +82,7 @@ static size_t carve_scc(void *base, int n, int m, SccWs *ws) {
     w.in_src = static_cast<int *>(take(4 * (M > 0 ? M : 1)));
     w.cursor = static_cast<int *>(take(4 * N));
     w.bsum = static_cast<int *>(take(4 * (N / kScanBlock + 2)));
-    w.color = static_cast<int *>(take(4 * N));
-    w.flags = static_cast<int *>(take(4 * N));
+    w.state = static_cast<unsigned long long *>(take(8 * N));
     w.piv = static_cast<int *>(take(4 * (3 * N + 1)));
     w.minv = static_cast<int *>(take(4 * N));
     for (int i = 0; i < 4; ++i) w.q[i] = static_cast<int *>(take(4 * N));
@@ -188,8 +195,7 @@ scc_init_kernel(int n, SccWs s, int *scc) {
         s.in_ptr[v] = 0;
         if (v < n) {
             s.cursor[v] = 0;
-            s.flags[v] = kActive;
-            s.color[v] = 3 * n;
+            s.state[v] = scc_key(3 * n);
             scc[v] = -1;
         }
     }
@@ -352,49 +358,80 @@ scc_iteration_kernel(const int *__restrict__ row_ptr, const int *__restrict__ co
             c->hcnt[1][k] = 0;
         }
     }
-    // 1. trimming: no active out- or in-neighbour in the own class
+    // 1. trimming: no active out- or in-neighbour in the own class (a state equal
+    //    to the vertex's own: no search has begun).  The rounds end when one takes
+    //    less than a sixteenth of what is active: a round costs the same however
+    //    little it takes, and the searches split the rest off as well.
+    int active = c->nrep ? c->nrep : n;   // (left by the last iteration, written at its end)
     for (int round = 0; round < kTrimRounds; ++round) {
         int removed = 0;
-        for (int v = gtid; v < n; v += stride) {
-            if (!(s.flags[v] & kActive)) continue;
-            const int cv = s.color[v];
-            bool out_ok = false, in_ok = false;
-            for (int e = row_ptr[v]; e < row_ptr[v + 1] && !out_ok; ++e) {
-                const int x = col[e];
-                out_ok = (s.flags[x] & kActive) && s.color[x] == cv;
+        for (int base = gtid; base < n; base += kTrimU * stride) {
+            unsigned long long my[kTrimU];
+            int e[kTrimU], e1[kTrimU], x[kTrimU];
+            bool ok[kTrimU];
+            // (the first out-, then the first in-neighbour of kTrimU vertices at once)
+#pragma unroll
+            for (int u = 0; u < kTrimU; ++u) {
+                const int v = base + u * stride;
+                my[u] = v < n ? s.state[v] : 0;
+                e[u] = my[u] ? row_ptr[v] : 0;
+                e1[u] = my[u] ? row_ptr[v + 1] : 0;
             }
-            for (int e = s.in_ptr[v]; out_ok && e < s.in_ptr[v + 1] && !in_ok; ++e) {
-                const int u = s.in_src[e];
-                in_ok = (s.flags[u] & kActive) && s.color[u] == cv;
+#pragma unroll
+            for (int u = 0; u < kTrimU; ++u) x[u] = e[u] < e1[u] ? col[e[u]] : -1;
+#pragma unroll
+            for (int u = 0; u < kTrimU; ++u) ok[u] = x[u] >= 0 && s.state[x[u]] == my[u];
+#pragma unroll
+            for (int u = 0; u < kTrimU; ++u) {
+                for (++e[u]; !ok[u] && e[u] < e1[u]; ++e[u]) ok[u] = s.state[col[e[u]]] == my[u];
+                const int v = base + u * stride;
+                e[u] = ok[u] ? s.in_ptr[v] : 0;
+                e1[u] = ok[u] ? s.in_ptr[v + 1] : 0;
             }
-            if (!out_ok || !in_ok) {
-                scc[v] = v;
-                s.flags[v] = 0;
-                ++removed;
+#pragma unroll
+            for (int u = 0; u < kTrimU; ++u) x[u] = e[u] < e1[u] ? s.in_src[e[u]] : -1;
+#pragma unroll
+            for (int u = 0; u < kTrimU; ++u) ok[u] = x[u] >= 0 && s.state[x[u]] == my[u];
+#pragma unroll
+            for (int u = 0; u < kTrimU; ++u) {
+                for (++e[u]; !ok[u] && e[u] < e1[u]; ++e[u]) ok[u] = s.state[s.in_src[e[u]]] == my[u];
+                const int v = base + u * stride;
+                if (my[u] && !ok[u]) {
+                    scc[v] = v;
+                    s.state[v] = 0;
+                    ++removed;
+                }
             }
         }
         bool ok;
         const int total = grid_sum_barrier(c, nb, removed, &ok);
         if (!ok) return;
-        if (total == 0) break;
+        if (total == 0 || total < active / 16) break;
+        active -= total;
     }
-    // 2. one pivot per class: its largest active vertex
-    for (int v = gtid; v < n; v += stride)
-        if (s.flags[v] & kActive) s.piv[s.color[v]] = -1;
+    // 2. one pivot per class: its largest active vertex (from the top, so that
+    //    most vertices of a large class find a larger one there already: a plain
+    //    read in place of an atomic on the one address they share)
+    for (int v = gtid; v < n; v += stride) {
+        const unsigned long long st = s.state[v];
+        if (st && load_volatile(&s.piv[scc_color(st)]) != -1) s.piv[scc_color(st)] = -1;
+    }
+    if (!grid_barrier(c, nb)) return;
+    for (int base = blockIdx.x * blockDim.x; base < n; base += stride) {
+        const int v = n - 1 - (base + (int)threadIdx.x);
+        const unsigned long long st = v >= 0 ? s.state[v] : 0;
+        const bool act = st && load_volatile(&s.piv[scc_color(st)]) < v;
+        warp_atomic_max(s.piv, act, act ? scc_color(st) : 0, v, lane);
+    }
     if (!grid_barrier(c, nb)) return;
     for (int base = blockIdx.x * blockDim.x; base < n; base += stride) {
         const int v = base + threadIdx.x;
-        const bool act = v < n && (s.flags[v] & kActive);
-        warp_atomic_max(s.piv, act, act ? s.color[v] : 0, v, lane);
-    }
-    if (!grid_barrier(c, nb)) return;
-    for (int base = blockIdx.x * blockDim.x; base < n; base += stride) {
-        const int v = base + threadIdx.x;
-        const bool pv = v < n && (s.flags[v] & kActive) && s.piv[s.color[v]] == v;
+        const unsigned long long st = v < n ? s.state[v] : 0;
+        const bool pv = st && s.piv[scc_color(st)] == v;
         bool hf = false, hb = false;
         if (pv) {
             s.minv[v] = INT_MAX;
-            s.flags[v] = kActive | kFw | kBw;
+            s.state[v] = st | kFw | kBw;
             hf = row_ptr[v + 1] - row_ptr[v] > kSccHeavy;
             hb = s.in_ptr[v + 1] - s.in_ptr[v] > kSccHeavy;
         }
@@ -445,12 +482,13 @@ scc_iteration_kernel(const int *__restrict__ row_ptr, const int *__restrict__ co
         for (int task = warp_id; task < ntf + ntb; task += nwarps) {
             const bool fwd = task < ntf;
             const int i = (fwd ? task : task - ntf) * kPer + grp;
-            const int bit = fwd ? kFw : kBw;
+            const unsigned long long bit = fwd ? kFw : kBw;
             const int *adj = fwd ? col : s.in_src;
-            int e = 0, e1 = 0, cu = 0;
+            int e = 0, e1 = 0;
+            unsigned long long cu = 0;
             if (i < (fwd ? nf : nbk)) {
                 const int u = fwd ? qf[i] : qb[i];
-                cu = s.color[u];
+                cu = s.state[u] & ~kReached;
                 e = (fwd ? row_ptr[u] : s.in_ptr[u]) + sub;
                 e1 = fwd ? row_ptr[u + 1] : s.in_ptr[u + 1];
             }
@@ -462,9 +500,9 @@ scc_iteration_kernel(const int *__restrict__ row_ptr, const int *__restrict__ co
                 if (more) {
                     x = adj[e];
                     e += LG;
-                    const int f = s.flags[x];
-                    if ((f & kActive) && !(f & bit) && s.color[x] == cu)
-                        take = !(atomicOr(&s.flags[x], bit) & bit);
+                    const unsigned long long f = s.state[x];
+                    if (!(f & bit) && (f & ~kReached) == cu)
+                        take = !(atomicOr(&s.state[x], bit) & bit);
                 }
                 push(fwd, take, x);
                 added += take;
@@ -475,9 +513,9 @@ scc_iteration_kernel(const int *__restrict__ row_ptr, const int *__restrict__ co
         for (int j = 0; j < nhf + nhb; ++j) {
             const bool fwd = j < nhf;
             const int u = fwd ? hqf[j] : hqb[j - nhf];
-            const int bit = fwd ? kFw : kBw;
+            const unsigned long long bit = fwd ? kFw : kBw;
             const int *adj = fwd ? col : s.in_src;
-            const int cu = s.color[u];
+            const unsigned long long cu = s.state[u] & ~kReached;
             int e = (fwd ? row_ptr[u] : s.in_ptr[u]) + gtid;
             const int e1 = fwd ? row_ptr[u + 1] : s.in_ptr[u + 1];
             for (;;) {
@@ -488,9 +526,9 @@ scc_iteration_kernel(const int *__restrict__ row_ptr, const int *__restrict__ co
                 if (more) {
                     x = adj[e];
                     e += stride;
-                    const int f = s.flags[x];
-                    if ((f & kActive) && !(f & bit) && s.color[x] == cu)
-                        take = !(atomicOr(&s.flags[x], bit) & bit);
+                    const unsigned long long f = s.state[x];
+                    if (!(f & bit) && (f & ~kReached) == cu)
+                        take = !(atomicOr(&s.state[x], bit) & bit);
                 }
                 push(fwd, take, x);
                 added += take;
@@ -509,22 +547,23 @@ scc_iteration_kernel(const int *__restrict__ row_ptr, const int *__restrict__ co
     // 4. split: reached both ways = the pivot's component
     for (int base = blockIdx.x * blockDim.x; base < n; base += stride) {
         const int v = base + threadIdx.x;
-        const int f = v < n ? s.flags[v] : 0;
-        const bool in = (f & kActive) && (f & kFw) && (f & kBw);
-        warp_atomic_min(s.minv, in, in ? s.piv[s.color[v]] : 0, v, lane);
+        const unsigned long long f = v < n ? s.state[v] : 0;
+        bool in = (f & kFw) && (f & kBw);
+        const int p = in ? s.piv[scc_color(f)] : 0;
+        in = in && load_volatile(&s.minv[p]) > v;
+        warp_atomic_min(s.minv, in, p, v, lane);
     }
     if (!grid_barrier(c, nb)) return;
     int still = 0;
     for (int v = gtid; v < n; v += stride) {
-        const int f = s.flags[v];
-        if (!(f & kActive)) continue;
-        const int p = s.piv[s.color[v]];
+        const unsigned long long f = s.state[v];
+        if (!f) continue;
+        const int p = s.piv[scc_color(f)];
         if ((f & kFw) && (f & kBw)) {
             scc[v] = s.minv[p];
-            s.flags[v] = 0;
+            s.state[v] = 0;
         } else {
-            s.color[v] = 3 * p + ((f & kFw) ? 1 : (f & kBw) ? 2 : 0);
-            s.flags[v] = kActive;
+            s.state[v] = scc_key(3 * p + ((f & kFw) ? 1 : (f & kBw) ? 2 : 0));
             ++still;
         }
     }
