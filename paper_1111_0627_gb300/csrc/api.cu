@@ -577,12 +577,19 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
         const long long cap = (opt && opt->max_iters > 0) ? opt->max_iters : 4LL * n + 64;
         const int k = launch_solve_team(row_ptr, col_idx, w, sign, n, m,
                                         opt ? opt->init_policy : nullptr, cap, out.cycle_out, ws, st);
-        if (k < 0) return OCM_ERR_CUDA;
-        launches += k;
-        int rc = read_ctrl(ws.ctrl, &h, st);
-        if (rc) return rc;
-        if (h.err) return map_err_bits(h.err);
-        if (!h.team_off) {   // (else a hub, which the general path spreads over the grid)
+        // (a cluster that the device cannot place -- too few SMs to share a GPC --
+        // or a hub, which the general path spreads over the grid: on as for others)
+        bool done = k > 0;
+        if (done) {
+            launches += k;
+            int rc = read_ctrl(ws.ctrl, &h, st);
+            if (rc) return rc;
+            if (h.err) return map_err_bits(h.err);
+            done = !h.team_off;
+        } else {
+            cudaGetLastError();
+        }
+        if (done) {
             if (h.not_converged) return OCM_ERR_NOT_CONVERGED;
             if (h.res_len < 1 || h.cnt[0] != h.res_len) return OCM_ERR_INTERNAL;
             if (outputs) {
