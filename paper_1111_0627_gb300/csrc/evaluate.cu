@@ -1518,6 +1518,22 @@ __global__ void extract_reset_kernel(Workspace ws) {
     ws.ctrl->walk_ok = 0;
 }
 
+// A short critical cycle: one thread follows the policy from its root, a
+// microsecond for two or three edges.  The candidates and the lifting take 8
+// launches and 50-80 us (2^20 vertices), most solves' cycles have 2-20 edges.
+constexpr int kChainLen = 48;
+
+__global__ void extract_chain_kernel(int L, Workspace ws, int *cycle_out) {
+    Ctrl *c = ws.ctrl;
+    const int r = c->res_root;
+    int y = r;
+    for (int k = 0; k < L; ++k) {
+        cycle_out[k] = ws.pi[y];
+        y = ws.succ[y];
+    }
+    c->cnt[0] = y == r ? L : 0;
+}
+
 // Extracts the critical cycle (root and length already in ctrl->res_*);
 // returns the number of kernel launches.  local_R: the block range size of
 // the two-level evaluation the loop used (0: the one-level evaluation, no
@@ -1525,6 +1541,11 @@ __global__ void extract_reset_kernel(Workspace ws) {
 int launch_extract(int n, int Lstar, Workspace ws, int *cycle_out, int grid, int local_R,
                    cudaStream_t st) {
     prof_begin(kProfExtract, st);
+    if (Lstar <= kChainLen) {
+        extract_chain_kernel<<<1, 1, 0, st>>>(Lstar, ws, cycle_out);
+        prof_end(kProfExtract, st);
+        return 1;
+    }
     extract_reset_kernel<<<1, 1, 0, st>>>(ws);
     int walk = 0;
     if (local_R > 0) {

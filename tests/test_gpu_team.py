@@ -53,7 +53,7 @@ def test_solve_wide_vertices(n, deg):
 
 
 @pytest.mark.parametrize("n,cycle", [(400, 48), (400, 49), (1000, 300), (3000, 2999), (10_000, 257),
-                                     (16_000, 16_000)])
+                                     (16_000, 16_000), (20_000, 48), (20_000, 49)])
 def test_solve_long_cycles_and_chains(n, cycle):
     """The heaviest cycle has the given length; the first policy leads into it
     by a chain of all other vertices, every one of which has a loop as well."""
