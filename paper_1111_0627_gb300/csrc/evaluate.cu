@@ -836,6 +836,9 @@ loop_control_kernel(Workspace ws, BatchState bs, int n, long long max_iters, int
             c->dirty_cnt = 0;
             c->changed = 0;
             c->switched = 0;
+            // (not at the next evaluation's start: where the walks settled every
+            // vertex its blocks pass no barrier before they raise it)
+            c->qmax = 0;
             if (more) {
                 c->nrep = kept;
                 c->old_roots = kept;
@@ -1181,7 +1184,6 @@ evaluate_kernel(int n, long long N2, int max_detect, int max_value, int stall_te
         bs.gbest[g] = 0;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         c->best = 0;   // (first used after a barrier, or by this block alone)
-        c->qmax = 0;
         if (all) c->nrep = 0;
         c->rounds_detect += 1;
         c->items_detect += n;
