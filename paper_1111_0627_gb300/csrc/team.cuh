@@ -213,9 +213,12 @@ static __device__ __forceinline__ int team_list_cycle(const Team<C> &tm, const T
 // looks for a cycle the samples missed, and a vertex that ends at such a root adds its steps
 // up again, to the first time its path meets it.
 
-// The seed phase; returns the roots listed.
+// The seed phase, after which `kept` old roots and the new ones are listed;
+// returns their number, the same in every thread (the shared counter may be
+// raised by those already walking).
 template <int C, bool SM>
-static __device__ __forceinline__ int team_seed(Team<C> &tm, const TeamGraph &g, JLS *st) {
+static __device__ __forceinline__ int team_seed(Team<C> &tm, const TeamGraph &g, JLS *st,
+                                                int kept) {
     const Workspace &ws = g.ws;
     const int i = g.n <= tm.W ? tm.tid : (int)((long long)tm.tid * g.n / tm.W);
     const int v = g.v0 + min(i, g.n - 1);
@@ -241,16 +244,16 @@ static __device__ __forceinline__ int team_seed(Team<C> &tm, const TeamGraph &g,
     if (cycle) team_list_cycle<C>(tm, g, cur, kTeamSeedSteps, &first);
     else if (s.J < 0 && len > 0) team_store<SM>(&st[v], JLS{s.J, len + s.len, S + s.S});
     const int fresh = tm.sum(first);
-    const int seeded = *reinterpret_cast<volatile int *>(&tm.sh->nrep);
+    const int seeded = kept + fresh;
     if (fresh) {
-        for (int k = seeded - fresh + tm.tid; k < seeded; k += tm.W) {
+        for (int k = kept + tm.tid; k < seeded; k += tm.W) {
             const int r = ws.cyc_root[g.v0 + k];
             team_store<SM>(&st[r], JLS{~r, 0, 0});
             ws.root_mark[r] = kRootOld;
         }
         tm.sync();
         // (tagged while the others go on)
-        for (int k = seeded - fresh + tm.tid; k < seeded; k += tm.W) {
+        for (int k = kept + tm.tid; k < seeded; k += tm.W) {
             const int r = ws.cyc_root[g.v0 + k];
             if (!team_tag_cycle(ws, r)) ws.root_mark[r] = kRootSeed;
         }
@@ -258,15 +261,16 @@ static __device__ __forceinline__ int team_seed(Team<C> &tm, const TeamGraph &g,
     return seeded;
 }
 
-// Both phases on one copy of the states; returns the vertices left open.
+// Both phases on one copy of the states, the first `kept` roots being listed
+// and settled; returns the vertices left open.
 template <int C, bool SM>
-static __device__ __forceinline__ int team_walk(Team<C> &tm, const TeamGraph &g) {
+static __device__ __forceinline__ int team_walk(Team<C> &tm, const TeamGraph &g, int kept) {
     const Workspace &ws = g.ws;
     const int lane = threadIdx.x & 31;
     JLS *st = g.st - g.v0;
     const int v1 = g.v0 + g.n;
     bool first = false;
-    const int seeded = team_seed<C, SM>(tm, g, st);
+    const int seeded = team_seed<C, SM>(tm, g, st, kept);
     const int root0 = seeded > 0 ? ws.cyc_root[g.v0] : -1;
     int left = 0;
     for (int base = g.v0 + tm.tid - lane; base < v1; base += tm.W) {
@@ -546,6 +550,7 @@ static __device__ bool team_evaluate(Team<C> &tm, const TeamGraph &g, TeamMode &
     const int n = g.n, v0 = g.v0;
     const int W = tm.W;
     if (mode.walk) {
+        int kept = 0;   // roots whose cycle no switch broke
         for (int base = tm.tid; base < n; base += kSU * W) {
             int m[kSU], sv[kSU], wv[kSU];   // (loads of kSU vertices in flight)
 #pragma unroll
@@ -566,13 +571,13 @@ static __device__ bool team_evaluate(Team<C> &tm, const TeamGraph &g, TeamMode &
                     ws.cyc_root[pos] = v;
                     ws.cid_of_root[v] = pos;
                     s = JLS{~v, 0, 0};
+                    ++kept;
                 }
                 if (m[u]) ws.root_mark[v] = keep ? kRootOld : 0;
                 g.st[i] = s;
             }
         }
-    tm.sync();
-        if (team_walk<C, SM>(tm, g) > 0) {
+        if (team_walk<C, SM>(tm, g, tm.sum(kept)) > 0) {
             mode.walk = false;
             mode.failed = true;
             if (tm.tid == 0) tm.sh->nrep = 0;
