@@ -930,7 +930,9 @@ static __device__ bool jump_resolve(int n, int F, bool all, int max_detect, int 
                 ws.jm[1][v] = f;
                 ws.rep[v] = ~s.J;
                 V[1][v] = s;
-                if (ratio) VT[0][v] = VT[1][v] = path_time(VT[0][v]);
+                // (a root settled by a walk from elsewhere has no time stored if
+                // its own walk gave up)
+                if (ratio) VT[0][v] = VT[1][v] = s.len > 0 ? path_time(VT[0][v]) : 0;
             }
         }
         block_append(LA, s_cnt, keep, v, lane);

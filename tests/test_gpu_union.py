@@ -44,3 +44,43 @@ def test_ratio_batch_of_many_graphs(G):
                for g, t in zip(graphs, times)]
     for rep in range(3):
         _check_batch(b, graphs, ocm.solve_batch(vp, rp, col, w, "max", transit=tt), oracles)
+
+
+@pytest.mark.parametrize("seed", range(3))
+def test_ratio_roots_settled_by_others(seed):
+    """Pairs that become cycles at the third evaluation, 16 to a warp, most of
+    which a warp gives up on; walks that come by from elsewhere settle some of
+    their roots all the same.  A root's value is 0 whoever settled it."""
+    rng = np.random.default_rng(9_200 + seed)
+    n, pairs, feeders = 120_000, 1000, 3000
+    a = 64 + 2 * np.arange(pairs)         # pairs (a, a + 1), neighbours in the vertex order
+    edges = [np.stack([np.arange(n), np.arange(n) // 3, rng.integers(-6, -1, n)], 1)]   # a tree
+    edges[0][0] = (0, 0, 0)               # ... to a loop of mean 0
+    high, low = n - 1, n - 2
+    edges[0][high], edges[0][low] = (high, 0, 500), (low, 0, -500)
+    edges[0][a] = np.stack([a, np.full(pairs, high), rng.integers(0, 50, pairs)], 1)
+    edges[0][a + 1] = np.stack([a + 1, np.full(pairs, low), rng.integers(0, 50, pairs)], 1)
+    c = n - 10 - feeders + np.arange(feeders)
+    edges[0][c] = np.stack([c, a[rng.permutation(feeders) % pairs], rng.integers(-9, 9, feeders)], 1)
+    edges.append(np.stack([a, a + 1, rng.integers(1, 9, pairs)], 1))
+    edges.append(np.stack([a + 1, a, rng.integers(1, 9, pairs)], 1))
+    e = np.concatenate(edges)
+    # (nothing of the tree leads through the pairs or the feeders)
+    inner = np.isin(e[:, 1], np.concatenate([a, a + 1, c])) & ~np.isin(e[:, 0], np.concatenate(
+        [a, a + 1, c]))
+    e[inner, 1] = 1
+    order = np.argsort(e[:, 0], kind="stable")
+    e = e[order].astype(np.int32)
+    rp = np.zeros(n + 1, np.int32)
+    rp[1:] = np.cumsum(np.bincount(e[:, 0], minlength=n))
+    col, w = np.ascontiguousarray(e[:, 1]), np.ascontiguousarray(e[:, 2])
+    t = rng.integers(1, 9, col.shape[0]).astype(np.int32)
+    init = rp[:-1].copy()
+    h = oracle.howard(rp, col, w, "max", init_policy=init, transit=t)
+    assert h.iterations >= 2
+    d = _dev(rp, col, w, init, t)
+    s = ocm.solve(*d[:3], "max", init_policy=d[3], transit=d[4], certificate=True)
+    assert (s.num, s.den, s.stats["iterations"]) == (h.num, h.den, h.iterations)
+    assert s.cycle.cpu().tolist() == h.cycle.tolist()
+    V = s.potential.cpu().numpy()
+    assert (V[a] == 0).all() and (V == h.V).all()
