@@ -569,8 +569,8 @@ int launch_csc(const int *row_ptr, const int *col, int n, int m, int *in_ptr, in
 int prepare_connect();
 int launch_connect(const int *row_ptr, const int *col, const int *w, int sign, int n,
                    Workspace ws, SingleWs sw, cudaStream_t st);
-void launch_outputs(int n, Workspace ws, BatchState bs, int64_t *eta_num, int32_t *eta_den, int64_t *potential,
-                    int32_t *policy, cudaStream_t st);
+void launch_outputs(int n, Workspace ws, BatchState bs, int64_t *eta_num, int32_t *eta_den,
+                    int64_t *potential, int32_t *policy, cudaStream_t st);
 void launch_backward(const int *cycle_edges, int cycle_len, const float *grad_lambda, int m,
                      float *grad_w, cudaStream_t st);
 

@@ -1574,17 +1574,29 @@ outputs_kernel(int n, Workspace ws, BatchState bs, int64_t *eta_num, int32_t *et
                int64_t *potential, int32_t *policy) {
     const int stride = gridDim.x * blockDim.x;
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        const JLS st = final_value(ws.jls[bs.G ? bs.gconv[bs.gid[v]] - 1 : 0], n, v);
-        int i = ws.cid_of_root[~st.J];
-        if (eta_num) eta_num[v] = ws.cyc_p[i];
-        if (eta_den) eta_den[v] = ws.cyc_q[i];
+        const int F = bs.G ? bs.gconv[bs.gid[v]] - 1 : 0;
+        const JLS st = final_value(ws.jls[F], n, v);
+        if (bs.G) {
+            // (the cycle table is the last step's: a graph that converged before
+            // it has no entries there; its states and records stay)
+            const int root = ~st.J, x = ws.succ[root], q = ws.rec[v].q;
+            const JLS sx = ws.jls[F][x];
+            const long long T = ws.transit ? ws.tpi[root] + path_time(ws.jt[F][x])
+                                           : 1 + (long long)sx.len;
+            if (eta_num) eta_num[v] = ((long long)ws.wpi[root] + sx.S) / (T / q);
+            if (eta_den) eta_den[v] = q;
+        } else {
+            const int i = ws.cid_of_root[~st.J];
+            if (eta_num) eta_num[v] = ws.cyc_p[i];
+            if (eta_den) eta_den[v] = ws.cyc_q[i];
+        }
         if (potential) potential[v] = ws.rec[v].V;
         if (policy) policy[v] = ws.pi[v];
     }
 }
 
-void launch_outputs(int n, Workspace ws, BatchState bs, int64_t *eta_num, int32_t *eta_den, int64_t *potential,
-                    int32_t *policy, cudaStream_t st) {
+void launch_outputs(int n, Workspace ws, BatchState bs, int64_t *eta_num, int32_t *eta_den,
+                    int64_t *potential, int32_t *policy, cudaStream_t st) {
     int blocks = (n + kThreads - 1) / kThreads;
     if (blocks > 8192) blocks = 8192;
     prof_begin(kProfExtract, st);

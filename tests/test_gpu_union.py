@@ -2,6 +2,8 @@
 disjoint union, walked and jumped together, with thousands of policy cycles in
 an evaluation, so that the cycle table is built by more than one block.  All
 results are exact integers, compared with the oracle's graph by graph."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -13,6 +15,7 @@ pytestmark = pytest.mark.gpu
 
 if torch.cuda.is_available():
     import paper_1111_0627_gb300 as ocm
+    from paper_1111_0627_gb300 import _native
 
 
 def _dev(*arrays):
@@ -84,3 +87,46 @@ def test_ratio_roots_settled_by_others(seed):
     assert s.cycle.cpu().tolist() == h.cycle.tolist()
     V = s.potential.cpu().numpy()
     assert (V[a] == 0).all() and (V == h.V).all()
+
+
+@pytest.mark.parametrize("ratio", [False, True], ids=["mean", "ratio"])
+def test_per_vertex_outputs_of_a_batch(ratio):
+    """Graphs that converge in different steps, among them some with several
+    cycles in the final policy: every vertex's value, cycle mean and policy
+    edge, through the C interface, are those of its graph solved alone."""
+    rng = np.random.default_rng(77 + ratio)
+    graphs = [synth.tiny_random(rng, int(rng.integers(1, 60)), max_extra=3, wlo=-30, whi=30,
+                                ring=k % 3 == 0) for k in range(150)]
+    graphs += [synth.ring_extra(3000, 0, 5, -100, 100, seed=8, tag=k, mode="max") for k in range(3)]
+    times = [rng.integers(1, 9, g.m).astype(np.int32) for g in graphs]
+    b = synth.concat(graphs)
+    N, M, G = b.row_ptr.shape[0] - 1, b.col_idx.shape[0], len(graphs)
+    vp, rp, col, w, tt = _dev(b.graph_vptr, b.row_ptr, b.col_idx, b.w, np.concatenate(times))
+    lib = _native.load()
+    out = {"eta_num": torch.zeros(N, dtype=torch.int64, device="cuda"),
+           "eta_den": torch.zeros(N, dtype=torch.int32, device="cuda"),
+           "potential": torch.zeros(N, dtype=torch.int64, device="cuda"),
+           "policy": torch.zeros(N, dtype=torch.int32, device="cuda")}
+    opt = _native.OcmOptions()
+    for k, x in out.items():
+        setattr(opt, k, x.data_ptr())
+    if ratio:
+        opt.transit = tt.data_ptr()
+    num = torch.zeros(G, dtype=torch.int64, device="cuda")
+    den, clen = (torch.zeros(G, dtype=torch.int32, device="cuda") for _ in range(2))
+    cyc = torch.zeros(N, dtype=torch.int32, device="cuda")
+    ws = torch.empty(lib.ocm_workspace_size_batch(G, N, M), dtype=torch.uint8, device="cuda")
+    rc = lib.ocm_solve_batch(vp.data_ptr(), rp.data_ptr(), col.data_ptr(), w.data_ptr(), G, N, M, 0,
+                             num.data_ptr(), den.data_ptr(), clen.data_ptr(), cyc.data_ptr(),
+                             ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream,
+                             ctypes.byref(opt), None)
+    assert rc == 0
+    got = {k: x.cpu().numpy() for k, x in out.items()}
+    for k, g in enumerate(graphs):
+        h = oracle.howard(g.row_ptr, g.col_idx, g.w, "max", transit=times[k] if ratio else None)
+        v0, v1 = int(b.graph_vptr[k]), int(b.graph_vptr[k + 1])
+        assert (int(num[k]), int(den[k])) == (h.num, h.den), k
+        assert (got["eta_num"][v0:v1] == h.eta_p).all(), k
+        assert (got["eta_den"][v0:v1] == h.eta_q).all(), k
+        assert (got["potential"][v0:v1] == h.V).all(), k
+        assert (got["policy"][v0:v1] - int(b.row_ptr[v0]) == h.policy).all(), k
