@@ -173,6 +173,8 @@ struct Ctrl {
     int old_roots;            // roots listed and settled before the walks
     int jump_rounds;
     int walk_fail;            // walks were dropped before in this solve
+    int walk_tries;           // how often they left too much,
+    int walk_pause;           // and the evaluations that jump before they are tried again
     int walk_deep;            // the next walks publish their parts (deep policies, evaluate.cu)
     unsigned long long depth_sum;   // path lengths of the policy just evaluated, of every eighth
     int depth_cnt;                  // block's vertices: their sum, and how many
@@ -183,8 +185,10 @@ struct Ctrl {
 // vertices unresolved are dropped, and every vertex goes to the jump rounds.
 // After that the number of detection rounds of a jump phase tells the depth (r
 // rounds: paths of at most about 2^(r - 1) steps), and the next evaluation
-// walks if it is at most kWalkRounds.  The first evaluation of a cold start
-// jumps: the heaviest edges form a random mapping, about sqrt(n) deep.
+// walks if it is at most kWalkRounds, the policy has no more cycles than are
+// settled ahead, and the failures before are long enough ago
+// (loop_control_kernel).  The first evaluation of a cold start jumps: the
+// heaviest edges form a random mapping, about sqrt(n) deep.
 constexpr int kWalkOffShift = 3;
 // Deep policies (an average path of more than kWalkDeep steps) walk with
 // published parts, up to kWalkDeepRounds.
@@ -193,7 +197,9 @@ constexpr int kWalkRounds = 9;
 constexpr int kWalkDeep = 48;
 constexpr int kWalkDeepRounds = 12;
 constexpr int kWalkDeepGraphs = 64;  // (of a batch: active graphs at most)
-constexpr int kSettleRoots = 1024;   // roots settled ahead of the walks at most
+// Roots settled ahead of the walks at most: one block does it, 16 rounds of a
+// few gathers at this number.
+constexpr int kSettleRoots = 8192;
 
 // The record pass marks the records it changes when the sweep before it
 // switched fewer than n >> kFrontierSwitchShift vertices, and the next sweep

@@ -785,81 +785,105 @@ walk_kernel(int n, Workspace ws, BatchState bs) {
 // It also prepares the counters the next evaluation starts from, and decides
 // whether its record pass marks the records it changes (frontier sweep) and
 // how it walks.
-// The first warp: the one-level evaluation's marked cycles that no switch broke
-// stay listed, and their roots are settled for the next evaluation.  The whole
-// block, where none stayed: the samples look for the new cycles.
+// Before that, the one-level evaluation's marked cycles that no switch broke
+// stay listed, and their roots are settled for the next evaluation; after it,
+// where none stayed, the samples look for the new cycles.
 __global__ void __launch_bounds__(kSampleThreads)
 loop_control_kernel(Workspace ws, BatchState bs, int n, long long max_iters, int use_cond,
                     cudaGraphConditionalHandle handle) {
     __shared__ int s_sample;
+    __shared__ int s_count[kSampleThreads / 32];
     Ctrl *c = ws.ctrl;
-    if (threadIdx.x < 32) {
-        int kept = 0;
-        const bool more = c->err == 0 && c->changed && (long long)c->iter + 1 < max_iters;
-        if (more && ws.walk && c->nrep <= kSettleRoots) {
-            JLS *next = ws.jls[(c->iter + 1) & 1];
-            const int tag = c->iter + 2;   // of the next evaluation
-            const int lane = threadIdx.x;
-            for (int base = 0; base < c->nrep; base += 32) {
-                const int r = base + lane < c->nrep ? ws.cyc_root[base + lane] : -1;
-                const bool keep =
-                    r >= 0 && (ws.root_mark[r] & 1) && !(bs.G && bs.gconv[bs.gid[r]]);
-                const unsigned m = __ballot_sync(0xffffffffu, keep);
-                if (keep) {
-                    const int pos = kept + __popc(m & ((1u << lane) - 1u));   // (<= base + lane)
-                    ws.cyc_root[pos] = r;
-                    ws.cid_of_root[r] = pos;
-                    ws.root_mark[r] = (tag << 1) | 1;
-                    next[r] = JLS{~r, 0, 0};
-                }
-                kept += __popc(m);
-                __syncwarp();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool more = c->err == 0 && c->changed && (long long)c->iter + 1 < max_iters;
+    const int K = c->nrep, iter = c->iter;
+    int kept = 0;
+    if (more && ws.walk && K <= kSettleRoots) {
+        JLS *next = ws.jls[(iter + 1) & 1];
+        const int tag = iter + 2;   // of the next evaluation
+        for (int base = 0; base < K; base += kSampleThreads) {
+            const int at = base + (int)threadIdx.x;
+            const int r = at < K ? ws.cyc_root[at] : -1;
+            const bool keep = r >= 0 && (ws.root_mark[r] & 1) && !(bs.G && bs.gconv[bs.gid[r]]);
+            const unsigned m = __ballot_sync(0xffffffffu, keep);
+            if (lane == 0) s_count[warp] = __popc(m);
+            __syncthreads();   // (the list is compacted in place, a block's worth at a time)
+            int pos = kept + __popc(m & ((1u << lane) - 1u));   // (<= at)
+            for (int w = 0; w < kSampleThreads / 32; ++w) {
+                if (w < warp) pos += s_count[w];
+                kept += s_count[w];
+            }
+            if (keep) {
+                ws.cyc_root[pos] = r;
+                ws.cid_of_root[r] = pos;
+                ws.root_mark[r] = (tag << 1) | 1;
+                next[r] = JLS{~r, 0, 0};
+            }
+            __syncthreads();
+        }
+    }
+    __syncthreads();   // (the fields read above change below)
+    if (threadIdx.x == 0) {
+        // the next step's cooperative launches count their barriers from zero
+        for (int i = 0; i < 2; ++i) {
+            c->bar[i].arrive = 0;
+            for (int j = 0; j < 4; ++j) {
+                c->bar[i].sum[j] = 0;
+                c->bar[i].sum2[j] = 0;
             }
         }
-        __syncwarp();
-        if (threadIdx.x == 0) {
-            // the next step's cooperative launches count their barriers from zero
-            for (int i = 0; i < 2; ++i) {
-                c->bar[i].arrive = 0;
-                for (int j = 0; j < 4; ++j) {
-                    c->bar[i].sum[j] = 0;
-                    c->bar[i].sum2[j] = 0;
-                }
-            }
-            c->switched_total += c->switched;
-            if (more) c->iter += 1;
-            else if (c->err == 0 && c->changed) c->not_converged = 1;
-            c->mark = c->frontier == 2 ||
-                      (c->frontier &&
-                       (long long)c->switched < ((long long)n >> kFrontierSwitchShift));
-            c->dirty_on = c->mark;
-            c->dirty_cnt = 0;
-            c->changed = 0;
-            c->switched = 0;
-            // (not at the next evaluation's start: where the walks settled every
-            // vertex its blocks pass no barrier before they raise it)
-            c->qmax = 0;
-            if (more) {
-                c->nrep = kept;
-                c->old_roots = kept;
-            }
-            // (the ratio's sums stay 0)
-            c->walk_deep = c->depth_sum > (unsigned long long)kWalkDeep * (unsigned)c->depth_cnt &&
-                           (bs.G == 0 || c->active_graphs <= kWalkDeepGraphs);
-            c->depth_sum = 0;
-            c->depth_cnt = 0;
-            if (c->walk_on && c->walk_left > (n >> kWalkOffShift)) {
-                c->walk_on = 0;
-                c->walk_fail = 1;
-            }
-            if (!c->walk_on)
-                c->walk_on = !c->walk_fail ||
-                             c->jump_rounds <= (c->walk_deep ? kWalkDeepRounds : kWalkRounds);
-            c->walk_left = 0;
-            c->loop_more = more ? 1 : 0;
-            s_sample = more && ws.walk && c->walk_on && kept == 0;
-            if (use_cond) cudaGraphSetConditional(handle, more ? 1u : 0u);
+        c->switched_total += c->switched;
+        if (more) c->iter += 1;
+        else if (c->err == 0 && c->changed) c->not_converged = 1;
+        c->mark = c->frontier == 2 ||
+                  (c->frontier &&
+                   (long long)c->switched < ((long long)n >> kFrontierSwitchShift));
+        c->dirty_on = c->mark;
+        c->dirty_cnt = 0;
+        c->changed = 0;
+        c->switched = 0;
+        // (not at the next evaluation's start: where the walks settled every
+        // vertex its blocks pass no barrier before they raise it)
+        c->qmax = 0;
+        // Walks need their roots settled ahead: with 100,000 cycles of three in
+        // 2^20 vertices a warp meets 32 of them, gives up after a few and has
+        // cost as much as the jump rounds that follow.  A single graph of more
+        // cycles than are settled ahead jumps (9.1 ms a solve, 11.5 with a walk
+        // tried each time; 5,000 cycles: 4.0 ms jumping, 3.6 walking, 4.9
+        // walking with 1,024 settled); a batch, each of whose warps meets one
+        // or two graphs, is tried.  Walks that left too much are tried again
+        // after 0, 1, 3, 7 .. evaluations, so that a policy that stays as it is
+        // pays for few; not counted where the deep walks had no root and did
+        // not start.
+        const bool failed = c->walk_on && c->walk_left > (n >> kWalkOffShift);
+        if (failed) {
+            c->walk_on = 0;
+            c->walk_fail = 1;
         }
+        if (failed && !(c->walk_deep && c->old_roots == 0)) {
+            c->walk_pause = (1 << c->walk_tries) - 1;
+            c->walk_tries = min(c->walk_tries + 1, 20);
+        } else if (!c->walk_on && c->walk_pause > 0) {
+            c->walk_pause -= 1;
+        }
+        // (the ratio's sums stay 0)
+        c->walk_deep = c->depth_sum > (unsigned long long)kWalkDeep * (unsigned)c->depth_cnt &&
+                       (bs.G == 0 || c->active_graphs <= kWalkDeepGraphs);
+        c->depth_sum = 0;
+        c->depth_cnt = 0;
+        if (!c->walk_on)
+            c->walk_on = !c->walk_fail
+                             ? bs.G || K <= kSettleRoots
+                             : c->walk_pause == 0 && K <= kSettleRoots &&
+                                   c->jump_rounds <= (c->walk_deep ? kWalkDeepRounds : kWalkRounds);
+        if (more) {
+            c->nrep = kept;
+            c->old_roots = kept;
+        }
+        c->walk_left = 0;
+        c->loop_more = more ? 1 : 0;
+        s_sample = more && ws.walk && c->walk_on && kept == 0;
+        if (use_cond) cudaGraphSetConditional(handle, more ? 1u : 0u);
     }
     __syncthreads();
     if (!s_sample) return;
