@@ -226,11 +226,14 @@ static __device__ bool radix_ranks(int K, const Workspace &ws, Ctrl *c, unsigned
 // (per graph for a batch), and the records {V, rank, q} the next sweep
 // gathers.  Called by every thread of a cooperative evaluation kernel.
 //
+// leave: what goes into the next evaluation's value buffer (evaluate_kernel).
 // LOCAL (the two-level evaluation): a vertex whose local path ends at an exit
 // holds its state to that exit, completed on the fly (final_value).
+enum : int { kLeaveNothing, kLeaveSteps, kLeaveStates };
 template <bool RATIO, bool LOCAL = false>
 static __device__ void evaluate_tail(int n, long long N2, int F, const Workspace &ws,
-                                     const BatchState &bs, long long *s_key) {
+                                     const BatchState &bs, long long *s_key,
+                                     int leave = kLeaveNothing) {
     Ctrl *c = ws.ctrl;
     const unsigned nblocks = gridDim.x;
     const int lane = threadIdx.x & 31;
@@ -446,6 +449,12 @@ static __device__ void evaluate_tail(int n, long long N2, int F, const Workspace
                 const int q = tab_q[i];
                 Rec rec;
                 const long long T = ratio ? path_time(ws.jt[F][v]) : (long long)st[u].len;
+                if (leave == kLeaveStates) {
+                    ws.jls[F ^ 1][v] = st[u];
+                    if (ratio) ws.jt[F ^ 1][v] = T;
+                } else if (leave == kLeaveSteps) {
+                    ws.jls[F ^ 1][v] = JLS{ws.succ[v], 1, (long long)ws.wpi[v]};
+                }
                 if (tally) {
                     depth += st[u].len;
                     ++resolved;
@@ -778,6 +787,14 @@ walk_kernel(int n, Workspace ws, BatchState bs) {
     }
 }
 
+// The evaluations that jump before the walks are tried again, as of the end of
+// this one: see loop_control_kernel.
+static __device__ __forceinline__ int walk_pause(const Ctrl *c, int n) {
+    if (c->walk_on)
+        return c->walk_left > (n >> kWalkOffShift) ? (1 << c->walk_tries) - 1 : 0;
+    return max(c->walk_pause - 1, 0);
+}
+
 // Ends a step: stop on an error or when no vertex switched (Howard's
 // termination test, Alg. 1), else advance the iteration index unless the
 // cap is reached.  With use_cond the decision also sets the WHILE node's
@@ -797,10 +814,24 @@ loop_control_kernel(Workspace ws, BatchState bs, int n, long long max_iters, int
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool more = c->err == 0 && c->changed && (long long)c->iter + 1 < max_iters;
     const int K = c->nrep, iter = c->iter;
+    JLS *next = ws.jls[(iter + 1) & 1];
+    const int tag = iter + 2;   // of the next evaluation
     int kept = 0;
-    if (more && ws.walk && K <= kSettleRoots) {
-        JLS *next = ws.jls[(iter + 1) & 1];
-        const int tag = iter + 2;   // of the next evaluation
+    if (more && ws.walk && K <= 32) {   // (any policy but the first ones: one warp, no barrier)
+        if (warp == 0) {
+            const int r = lane < K ? ws.cyc_root[lane] : -1;
+            const bool keep = r >= 0 && (ws.root_mark[r] & 1) && !(bs.G && bs.gconv[bs.gid[r]]);
+            const unsigned m = __ballot_sync(0xffffffffu, keep);
+            if (keep) {
+                const int pos = __popc(m & ((1u << lane) - 1u));
+                ws.cyc_root[pos] = r;
+                ws.cid_of_root[r] = pos;
+                ws.root_mark[r] = (tag << 1) | 1;
+                next[r] = JLS{~r, 0, 0};
+            }
+            kept = __popc(m);
+        }
+    } else if (more && ws.walk && K <= kSettleRoots) {
         for (int base = 0; base < K; base += kSampleThreads) {
             const int at = base + (int)threadIdx.x;
             const int r = at < K ? ws.cyc_root[at] : -1;
@@ -852,26 +883,22 @@ loop_control_kernel(Workspace ws, BatchState bs, int n, long long max_iters, int
         // tried each time; 5,000 cycles: 4.0 ms jumping, 3.6 walking, 4.9
         // walking with 1,024 settled); a batch, each of whose warps meets one
         // or two graphs, is tried.  Walks that left too much are tried again
-        // after 0, 1, 3, 7 .. evaluations, so that a policy that stays as it is
-        // pays for few; not counted where the deep walks had no root and did
-        // not start.
-        const bool failed = c->walk_on && c->walk_left > (n >> kWalkOffShift);
-        if (failed) {
+        // after 0, 1, 3, 7 .. evaluations, counted from the last that did not,
+        // so that a policy that stays too deep pays for few.
+        c->walk_pause = walk_pause(c, n);
+        if (c->walk_on && c->walk_left <= (n >> kWalkOffShift)) {
+            c->walk_tries = 0;
+        } else if (c->walk_on) {
             c->walk_on = 0;
             c->walk_fail = 1;
-        }
-        if (failed && !(c->walk_deep && c->old_roots == 0)) {
-            c->walk_pause = (1 << c->walk_tries) - 1;
             c->walk_tries = min(c->walk_tries + 1, 20);
-        } else if (!c->walk_on && c->walk_pause > 0) {
-            c->walk_pause -= 1;
         }
         // (the ratio's sums stay 0)
         c->walk_deep = c->depth_sum > (unsigned long long)kWalkDeep * (unsigned)c->depth_cnt &&
                        (bs.G == 0 || c->active_graphs <= kWalkDeepGraphs);
         c->depth_sum = 0;
         c->depth_cnt = 0;
-        if (!c->walk_on)
+        if (!c->walk_on && !c->carry)   // (carry: certain to jump, see evaluate_kernel)
             c->walk_on = !c->walk_fail
                              ? bs.G || K <= kSettleRoots
                              : c->walk_pause == 0 && K <= kSettleRoots &&
@@ -919,10 +946,17 @@ void launch_walk_seed(int n, Workspace ws, cudaStream_t st) {
 // are off): detection by window minima, then values, as described at the top
 // of the file; every final state ends in jls[F] (times in jt[F]).  Scratch:
 // the 16-byte scratch is the other value buffer.  Returns false on an error or
-// when a grid barrier gave up (recorded in the control block).
+// when a grid barrier gave up (recorded in the control block); *rounds: the
+// detection rounds.
+//   carry: buffer F holds the last evaluation's final state of every vertex that
+// did not switch since, a step {J >= 0} of those that did (evaluate_kernel).
+// All vertices take part in the detection, whose window minima carry a second
+// bit: a vertex of the window switched.  A vertex without one on its whole path
+// and cycle keeps its state.
 template <bool RATIO>
-static __device__ bool jump_resolve(int n, int F, bool all, int max_detect, int max_value,
-                                    const Workspace &ws, const BatchState &bs, int *s_cnt) {
+static __device__ bool jump_resolve(int n, int F, bool all, bool carry, int max_detect,
+                                    int max_value, const Workspace &ws, const BatchState &bs,
+                                    int *s_cnt, int *rounds) {
     Ctrl *c = ws.ctrl;
     constexpr bool ratio = RATIO;   // optimal cycle ratio: times ride along
     const unsigned nblocks = gridDim.x;
@@ -934,54 +968,55 @@ static __device__ bool jump_resolve(int n, int F, bool all, int max_detect, int 
     int *LA = ws.list[0] + lo, *LB = ws.list[1] + lo;
     JLS *V[2] = {ws.jls[F], reinterpret_cast<JLS *>(ws.scratch16)};
     long long *VT[2] = {ws.jt[F], ws.jt[F ^ 1]};
+    int *LC = ws.list[2] + lo;   // (what the walks left; needed again for the values)
     if (threadIdx.x == 0) *s_cnt = 0;
     __syncthreads();
-    // ---- the worklist; settled vertices are resolved in both buffers
-    for (int i0 = 0; i0 < hi - lo; i0 += blockDim.x) {
-        const int i = i0 + threadIdx.x;
-        const int v = lo + i;
-        bool keep = false;
-        // batched: vertices of converged graphs keep everything
-        if (i < hi - lo && !(bs.G && bs.gconv[bs.gid[v]])) {
-            const JLS s = all ? JLS{0, 0, 0} : V[0][v];
-            if (s.J >= 0) {
-                keep = true;
-                // (no walk wrote the next evaluation's step)
-                if (all) ws.jls[F ^ 1][v] = JLS{ws.succ[v], 1, (long long)ws.wpi[v]};
-            } else {
-                const JM f{s.J, 0};
-                ws.jm[0][v] = f;
-                ws.jm[1][v] = f;
-                ws.rep[v] = ~s.J;
-                V[1][v] = s;
-                // (a root settled by a walk from elsewhere has no time stored if
-                // its own walk gave up)
-                if (ratio) VT[0][v] = VT[1][v] = s.len > 0 ? path_time(VT[0][v]) : 0;
+    int cnt0 = hi - lo;
+    // ---- the worklist; vertices the walks settled are resolved (in both
+    // buffers) and keep their state: rep = ~root, as for the unchanged ones below.
+    // (All vertices: no list, and no barrier, since round 0 starts from succ.)
+    if (!all) {
+        for (int i0 = 0; i0 < hi - lo; i0 += blockDim.x) {
+            const int i = i0 + threadIdx.x;
+            const int v = lo + i;
+            bool keep = false;
+            // batched: vertices of converged graphs keep everything
+            if (i < hi - lo && !(bs.G && bs.gconv[bs.gid[v]])) {
+                const JLS s = V[0][v];
+                if (s.J >= 0) {
+                    keep = true;
+                    ws.jm[0][v] = JM{ws.succ[v], v | INT_MIN};
+                } else {
+                    const JM f{s.J, 0};
+                    ws.jm[0][v] = f;
+                    ws.jm[1][v] = f;
+                    ws.rep[v] = s.J;
+                    // (a root settled by a walk from elsewhere has no time stored
+                    // if its own walk gave up)
+                    if (ratio) VT[0][v] = s.len > 0 ? path_time(VT[0][v]) : 0;
+                }
             }
+            block_append(LA, s_cnt, keep, v, lane);
         }
-        block_append(LA, s_cnt, keep, v, lane);
+        __syncthreads();
+        cnt0 = *s_cnt;
+        __syncthreads();
+        if (threadIdx.x == 0) *s_cnt = 0;
+        for (int i = threadIdx.x; i < cnt0; i += blockDim.x) LC[i] = LA[i];
+        if (!grid_barrier(c, nblocks)) return false;
     }
-    __syncthreads();
-    const int cnt0 = *s_cnt;
-    __syncthreads();
-    if (threadIdx.x == 0) *s_cnt = 0;
-    // (the list of unfinished vertices is needed again for the values)
-    int *LC = ws.list[2] + lo;
-    for (int i = threadIdx.x; i < cnt0; i += blockDim.x) {
-        const int v = LA[i];
-        LC[i] = v;
-        ws.jm[0][v] = JM{ws.succ[v], v};
-    }
-    if (!grid_barrier(c, nblocks)) return false;
+    // did v switch since the states in buffer F were found?
+    auto switched = [&](int v) -> int { return carry && V[0][v].J < 0 ? 0 : INT_MIN; };
 
     // ------------------------------------------------------------ detect
-    // State: unresolved {J >= 0, window minimum}; resolved {~root, 0}.
+    // State: unresolved {J >= 0, window minimum | switched << 31}; resolved {~root, switched}.
     int cnt = cnt0;
     for (int r = 0;; ++r) {
         const JM *in = ws.jm[r & 1];
         JM *out = ws.jm[(r + 1) & 1];
         int *lin = (r & 1) ? LB : LA;
         int *lout = (r & 1) ? LA : LB;
+        const bool first = all && r == 0;
         int pend = 0, kept = 0;
         for (int i0 = 0; i0 < cnt; i0 += kU * blockDim.x) {
             int item[kU];
@@ -990,19 +1025,23 @@ static __device__ bool jump_resolve(int n, int F, bool all, int max_detect, int 
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
                 const int i = i0 + u * blockDim.x + threadIdx.x;
-                item[u] = i < cnt ? lin[i] : INT_MIN;
+                item[u] = i >= cnt ? INT_MIN : first ? lo + i : lin[i];
+                if (first && i < cnt && bs.G && bs.gconv[bs.gid[lo + i]]) item[u] = INT_MIN;
             }
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
                 const int it = item[u];
                 if (it == INT_MIN) continue;
                 const int v = it < 0 ? ~it : it;
-                s[u] = in[v];
+                s[u] = first ? JM{ws.succ[v], v | switched(v)} : in[v];
                 ap[u] = (r > 0 && it >= 0) ? ws.aprev[v] : -1;
             }
 #pragma unroll
-            for (int u = 0; u < kU; ++u)
-                if (item[u] != INT_MIN && item[u] >= 0) t[u] = in[s[u].J];
+            for (int u = 0; u < kU; ++u) {
+                if (item[u] == INT_MIN || item[u] < 0) continue;
+                const int J = s[u].J;
+                t[u] = first ? JM{ws.succ[J], J | switched(J)} : in[J];
+            }
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
                 const int it = item[u];
@@ -1013,20 +1052,23 @@ static __device__ bool jump_resolve(int n, int F, bool all, int max_detect, int 
                     if (it < 0) {
                         out[v] = s[u];        // resolved last round: copy forward
                     } else {
-                        int root = -1;
+                        const int sm = s[u].M & INT_MAX, tm = t[u].M & INT_MAX;
+                        int root = -1, sw = (int)((unsigned)s[u].M >> 31);
                         if (t[u].J < 0) {
                             root = ~t[u].J;   // target resolved: it lies on v's path
-                        } else if (r > 0 && t[u].M == ap[u]) {
-                            root = ap[u];     // smallest vertex of the cycle
+                            sw |= t[u].M;
+                        } else if (r > 0 && tm == ap[u]) {
+                            root = tm;        // smallest vertex of the cycle
+                            sw |= (int)((unsigned)t[u].M >> 31);
                         } else {
                             // (round 0: J_0 = succ, M_0(v) = v, no test yet)
-                            out[v] = JM{t[u].J, min(s[u].M, t[u].M)};
-                            ws.aprev[v] = t[u].M;
+                            out[v] = JM{t[u].J, min(sm, tm) | ((s[u].M | t[u].M) & INT_MIN)};
+                            ws.aprev[v] = tm;
                             keep = true;
                         }
                         if (root >= 0) {
-                            out[v] = JM{~root, 0};
-                            ws.rep[v] = root;
+                            out[v] = JM{~root, sw};
+                            ws.rep[v] = sw ? root : ~root;
                             resolved = true;
                             is_root = (root == v);
                         }
@@ -1051,7 +1093,7 @@ static __device__ bool jump_resolve(int n, int F, bool all, int max_detect, int 
         const int left = grid_sum2_barrier(c, nblocks, pend, kept, &still, &ok);
         if (!ok) return false;
         if (left == 0 || still == 0) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) c->jump_rounds = r + 1;
+            *rounds = r + 1;
             break;
         }
         if (r + 1 >= max_detect) {
@@ -1061,8 +1103,8 @@ static __device__ bool jump_resolve(int n, int F, bool all, int max_detect, int 
     }
 
     // ------------------------------------------------------------ values
-    // Roots are final at once, as is a vertex whose successor is a root; the
-    // rest jump until they meet a final state.
+    // Roots are final at once, as is a vertex whose successor is a root or keeps
+    // its state (rep = ~root); the rest jump until they meet a final state.
     cnt = 0;
     int left0 = 0;
     {
@@ -1070,10 +1112,12 @@ static __device__ bool jump_resolve(int n, int F, bool all, int max_detect, int 
         for (int i0 = 0; i0 < cnt0; i0 += blockDim.x) {
             const int i = i0 + threadIdx.x;
             bool keep = false;
-            int v = 0;
+            int v = 0, root = -1;
             if (i < cnt0) {
-                v = LC[i];
-                const int root = ws.rep[v];
+                v = all ? lo + i : LC[i];
+                if (!(all && bs.G && bs.gconv[bs.gid[v]])) root = ws.rep[v];
+            }
+            if (root >= 0) {
                 JLS st;
                 long long T = 0;
                 bool fin = true;
@@ -1081,9 +1125,15 @@ static __device__ bool jump_resolve(int n, int F, bool all, int max_detect, int 
                     st = JLS{~v, 0, 0};
                 } else {
                     const int sv = ws.succ[v];
-                    fin = (ws.rep[sv] == sv);
-                    st = JLS{fin ? ~sv : sv, 1, (long long)ws.wpi[v]};
+                    const int rs = ws.rep[sv];
+                    fin = rs < 0 || rs == sv;
+                    st = JLS{rs == sv ? ~sv : sv, 1, (long long)ws.wpi[v]};
                     if (ratio) T = ws.tpi[v];
+                    if (rs < 0) {
+                        const JLS sf = V[0][sv];
+                        st = JLS{sf.J, 1 + sf.len, st.S + sf.S};
+                        if (ratio) T += path_time(VT[0][sv]);
+                    }
                 }
                 V[0][v] = st;
                 if (fin) V[1][v] = st;
@@ -1205,22 +1255,44 @@ evaluate_kernel(int n, long long N2, int max_detect, int max_value, int stall_te
     const int left = c->walk_left;
     // (walks that were cut short may have settled a root whose own walk, which
     // lists it, never ran: everything is resolved again)
-    const bool all = !c->walk_on || left > (n >> kWalkOffShift);
+    const bool failed = c->walk_on && left > (n >> kWalkOffShift);
+    const bool all = !c->walk_on || failed;
+    const bool carry = all && c->carry;   // (rewritten below, after a barrier)
     for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < bs.G; g += gridDim.x * blockDim.x)
         bs.gbest[g] = 0;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         c->best = 0;   // (first used after a barrier, or by this block alone)
-        if (all) c->nrep = 0;
+        if (all) c->nrep = 0;   // (first raised after a barrier: round 0 finds no root)
         c->rounds_detect += 1;
         c->items_detect += n;
     }
     __syncthreads();
     // (test only: wait for one block more than exists, so the wait expires)
     if (stall_test && !grid_barrier(c, nblocks + 1u)) return;
+    // What the record pass leaves in the next evaluation's buffer, where the
+    // sweep's switches then put their steps: nothing where the walks have put
+    // every vertex's step; the steps; or, where the next evaluation is sure to
+    // jump, the final states, which a vertex whose path sees no switch then keeps.
+    // Deep policies change little a step: 300,000 vertices, paths of up to 10,000,
+    // 205 iterations, take 32.5 ms (38.8 with all values found anew and a walk
+    // tried each time); 2,000,000 134 (165).
+    int leave = kLeaveNothing;
     if (all || left > 0) {
-        if (!jump_resolve<RATIO>(n, F, all, max_detect, max_value, ws, bs, &s_cnt)) return;
+        int rounds = 0;
+        if (!jump_resolve<RATIO>(n, F, all, carry, max_detect, max_value, ws, bs, &s_cnt, &rounds))
+            return;
+        const bool dropped = c->walk_fail || failed;
+        const bool stays =
+            all && (load_volatile(&c->nrep) > kSettleRoots
+                        ? dropped || bs.G == 0
+                        : dropped && (rounds > kWalkDeepRounds || walk_pause(c, n) > 0));
+        if (all) leave = stays ? kLeaveStates : kLeaveSteps;
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            c->jump_rounds = rounds;
+            c->carry = stays ? 1 : 0;
+        }
     }
-    evaluate_tail<RATIO>(n, N2, F, ws, bs, s_key);
+    evaluate_tail<RATIO>(n, N2, F, ws, bs, s_key, leave);
 }
 
 // SMs of the current device.
