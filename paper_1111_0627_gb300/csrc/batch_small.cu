@@ -122,7 +122,8 @@ small_graph_kernel(const int *__restrict__ row_ptr, const int *__restrict__ col,
         if (tm.tid == 0) {
             if (capped) c->not_converged = 1;
             if (ok) {
-                const unsigned long long packed = tm.sh->best;
+                const unsigned long long packed =
+                    *reinterpret_cast<volatile unsigned long long *>(tg.best);
                 const int root = INT_MAX - (int)(unsigned)(packed & 0xffffffffu);
                 const int i = ws.cid_of_root[root];
                 bs.gbest[g] = packed;

@@ -196,7 +196,7 @@ solve_team_kernel(const int *__restrict__ row_ptr, const int *__restrict__ col,
             : team_iterate<C, false>(tm, g, init != nullptr, max_iters, &it, &switched, &capped);
     if (tm.tid == 0 && capped) c->not_converged = 1;
     if (ok) {
-        const unsigned long long packed = tm.sh->best;
+        const unsigned long long packed = *reinterpret_cast<volatile unsigned long long *>(g.best);
         const int r = INT_MAX - (int)(unsigned)(packed & 0xffffffffu);
         const int i = ws.cid_of_root[r];
         const int L = ws.cyc_L[i];

@@ -49,7 +49,6 @@ struct TeamShared {
     int nrep;
     int task;
     int K;
-    unsigned long long best;
 };
 
 template <int C>
@@ -130,6 +129,9 @@ struct TeamGraph {
     Rec *old;             // the records kept until the next evaluation
     unsigned *dirty;      // n bits: records the last evaluation changed (nullptr: no room)
     unsigned *bits;       // bitmaps of the jump rounds (nullptr: no trimming)
+    // the best cycle's (rank, INT_MAX - root).  In global memory: a 64-bit maximum
+    // in another block's shared memory lost updates (32-bit counts there do not).
+    unsigned long long *best;
     Workspace ws;
 };
 
@@ -540,7 +542,7 @@ struct TeamMode {
 
 // Policy evaluation: states, cycle table, records {V, rank, q} (with mark: the
 // bits of those that change; *n_dirty counts them).  The cycle records sit at
-// [v0, v0 + K); the best (rank, INT_MAX - root) is in tm.sh->best.  Returns
+// [v0, v0 + K); the best (rank, INT_MAX - root) is in *g.best.  Returns
 // false on an error (recorded in the control block).  tm.sh->nrep is 0 and
 // every team thread is past a barrier when it is called.
 template <int C, bool SM>
@@ -611,21 +613,25 @@ static __device__ bool team_evaluate(Team<C> &tm, const TeamGraph &g, TeamMode &
         ws.cyc_q[i] = (int)(L / d);
         ws.cyc_L[i] = (int)L;
         if (K > 1) ws.cyc_key[i] = mean_key(Wc / d, L / d, N2);
-        else tm.sh->best = (unsigned)(INT_MAX - r);
+        else *g.best = (unsigned)(INT_MAX - r);
     }
     if (mark)
         for (int i = tm.tid; i < (n + 31) / 32; i += W) g.dirty[i] = 0u;
-    if (K > 1 && tm.tid == 0) tm.sh->best = 0;
+    if (K > 1 && tm.tid == 0) *g.best = 0;
     tm.sync();
     if (K > 1) {
+        unsigned long long top = 0;
         for (int i = v0 + tm.tid; i < v0 + K; i += W) {
             const long long key = ws.cyc_key[i];
             int rank = 0;
             for (int j = v0; j < v0 + K; ++j) rank += ws.cyc_key[j] < key;
             ws.cyc_rank[i] = rank;
-            atomicMax(&tm.sh->best, ((unsigned long long)(unsigned)rank << 32) |
-                                        (unsigned)(INT_MAX - ws.cyc_root[i]));
+            top = max(top, ((unsigned long long)(unsigned)rank << 32) |
+                               (unsigned)(INT_MAX - ws.cyc_root[i]));
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+        if ((threadIdx.x & 31) == 0 && top) atomicMax(g.best, top);
         tm.sync();
     }
     // ---- materialise the records the sweep gathers
@@ -802,7 +808,7 @@ static __device__ __forceinline__ TeamGraph team_place(unsigned char *dyn, const
                                                        int v0, int n, const Workspace &ws,
                                                        int room, bool *in_shared) {
     TeamGraph g{row_ptr, col, w, sign, v0, n, ws.jls[0] + v0, ws.rec + v0, ws.rec + v0,
-                nullptr, nullptr, ws};
+                nullptr, nullptr, reinterpret_cast<unsigned long long *>(ws.recp + v0), ws};
     *in_shared = false;
     const long long nw = (n + 31) / 32;
     const long long d = ((C == 1 ? nw : 0) * 4 + 15) / 16 * 16;   // the frontier bitmap

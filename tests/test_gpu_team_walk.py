@@ -101,3 +101,27 @@ def test_given_policies_as_a_batch(shape):
             assert (int(s.num[k]), int(s.den[k])) == (h.num, h.den), (rep, k)
             assert (s.cycle(k).cpu() - e0[k]).tolist() == h.cycle.tolist(), (rep, k)
         assert s.stats["iterations"] == max(h.iterations for h in oracles)
+
+
+@pytest.mark.parametrize("n,K", [(512, 127), (512, 128), (1024, 255), (1024, 256), (1024, 512),
+                                 (1024, 513), (1024, 1024), (4096, 2048), (4096, 2049), (9000, 4100)])
+def test_best_of_many_cycles(n, K):
+    """K loops with many equal weights and a few better cycles, in blocks and in
+    clusters, whose blocks find the best of them together."""
+    rng = np.random.default_rng(n + K)
+    name = rng.permutation(n)
+    edges = []
+    for v in range(n):
+        if v < K:
+            edges.append((int(name[v]), int(name[v]), int(rng.integers(0, 40))))
+        else:
+            edges += [(int(name[v]), int(name[t]), int(rng.integers(0, 100)))
+                      for t in rng.integers(0, n, 3)] + [(int(name[v]), int(name[v - 1]), 0)]
+    g = synth.from_edges(n, edges, "max", "loops")
+    h = oracle.howard(g.row_ptr, g.col_idx, g.w, g.mode)
+    s = ocm.solve(*_dev(g.row_ptr, g.col_idx, g.w), g.mode, certificate=True)
+    assert s.stats["launches"] <= 2 and s.stats["cycles"] >= K
+    assert (s.num, s.den, s.stats["iterations"]) == (h.num, h.den, h.iterations)
+    assert s.cycle.cpu().tolist() == h.cycle.tolist()
+    assert (s.potential.cpu().numpy() == h.V).all()
+    assert (s.eta_num.cpu().numpy() == h.eta_p).all()
