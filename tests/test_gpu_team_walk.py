@@ -103,11 +103,12 @@ def test_given_policies_as_a_batch(shape):
         assert s.stats["iterations"] == max(h.iterations for h in oracles)
 
 
-@pytest.mark.parametrize("n,K", [(512, 127), (512, 128), (1024, 255), (1024, 256), (1024, 512),
+@pytest.mark.parametrize("n,K", [(512, 256), (1024, 511), (1024, 512), (4096, 510), (4096, 511),
                                  (1024, 513), (1024, 1024), (4096, 2048), (4096, 2049), (9000, 4100)])
 def test_best_of_many_cycles(n, K):
     """K loops with many equal weights and a few better cycles, in blocks and in
-    clusters, whose blocks find the best of them together."""
+    clusters, whose blocks find the best of them together; K on both sides of
+    the numbers at which one thread ranks a cycle, or several do."""
     rng = np.random.default_rng(n + K)
     name = rng.permutation(n)
     edges = []
