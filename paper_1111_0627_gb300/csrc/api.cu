@@ -568,6 +568,7 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
     const int req_kind = opt ? opt->sweep_kind : OCM_SWEEP_DEFAULT;
     const bool outputs =
         opt && (opt->eta_num || opt->eta_den || opt->potential || opt->policy);
+    bool row_checked = false;
     // A small graph with no form asked for: the whole solve by one block or
     // cluster.  (A host-driven or profiled loop, and the fallback to one, keep
     // the launch per step.)
@@ -578,7 +579,8 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
         const int k = launch_solve_team(row_ptr, col_idx, w, sign, n, m,
                                         opt ? opt->init_policy : nullptr, cap, out.cycle_out, ws, st);
         // (a cluster that the device cannot place -- too few SMs to share a GPC --
-        // or a hub, which the general path spreads over the grid: on as for others)
+        // or a hub, which the general path spreads over the grid: on as for others,
+        // after the hub's row_ptr has been checked)
         bool done = k > 0;
         if (done) {
             launches += k;
@@ -586,6 +588,7 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
             if (rc) return rc;
             if (h.err) return map_err_bits(h.err);
             done = !h.team_off;
+            row_checked = !done;
         } else {
             cudaGetLastError();
         }
@@ -625,13 +628,17 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
                                                                            : 1;
     ctrl_init_kernel<<<1, 1, 0, st>>>(ws.ctrl, wait_ns, frontier, local_chunks,
                                       opt && opt->init_policy ? 1 : 0);
-    launch_check_row_ptr(row_ptr, n, m, ws.ctrl, st);
-    launches += 2;
-    if (bs) launches += launch_batch_prepare(n, m, b, ws, st);
-    if (cudaGetLastError() != cudaSuccess) return OCM_ERR_CUDA;
-    int rc = read_ctrl(ws.ctrl, &h, st);
-    if (rc) return rc;
-    if (h.err) return map_err_bits(h.err);
+    launches += 1;
+    int rc = OCM_OK;
+    if (!row_checked) {
+        launch_check_row_ptr(row_ptr, n, m, ws.ctrl, st);
+        launches += 1;
+        if (bs) launches += launch_batch_prepare(n, m, b, ws, st);
+        if (cudaGetLastError() != cudaSuccess) return OCM_ERR_CUDA;
+        rc = read_ctrl(ws.ctrl, &h, st);
+        if (rc) return rc;
+        if (h.err) return map_err_bits(h.err);
+    }
 
     phase("ocm:init_policy");
     // 2. degree classes of the improvement sweep (and the heavy vertices), then
