@@ -8,7 +8,9 @@ blocks of ``sweep_threads``.  Which combination is fastest depends on the
 degree distribution and on how local the targets are, so :func:`tune` runs
 one full solve per candidate on the caller's graph, reads the sweep kernels'
 time from the library's own CUDA-event instrumentation (``ocm_profile_*``),
-and keeps the fastest.  Results are cached per graph signature (size and
+and keeps the fastest.  A small graph that the library solves in one launch by
+default keeps the default where the whole solve is faster so (any of these
+parameters, and the instrumentation, take the launch per step).  Results are cached per graph signature (size and
 degree buckets) in a JSON table (``OCM_TUNE_FILE``, default
 ``~/.cache/ocm_gb300/tune.json``); ``solve(..., tune=True)`` looks the
 signature up.  The solver's results never depend on these parameters -- only
@@ -30,6 +32,7 @@ TILES, CLASSES, WINDOW = 2, 1, 3   # OCM_SWEEP_TILES, _CLASSES, _WINDOW (include
 CANDIDATES = ([(TILES, epl, thr) for epl in (4, 8) for thr in (64, 128, 256)] +
               [(CLASSES, epl, thr) for epl in (2, 4, 8, 16, 32) for thr in (128, 256, 512)] +
               [(WINDOW, epl, 512) for epl in (2, 4, 8, 16)])
+ONE_LAUNCH_N = 1 << 14   # largest graph solved in one launch (csrc/solve_team.cu)
 SWEEP_CLASS = 1       # profiling class of the improvement sweep (include/ocm.h)
 _lock = threading.Lock()
 
@@ -72,13 +75,30 @@ def lookup(row_ptr: torch.Tensor) -> tuple[int, int, int] | None:
         entry = _load_table().get(signature(row_ptr))
     if not entry or "sweep_kind" not in entry:
         return None
+    # (a table written before small graphs were solved in one launch)
+    if row_ptr.numel() - 1 <= ONE_LAUNCH_N and "solve_ms" not in entry:
+        return None
     return int(entry["sweep_kind"]), int(entry["edges_per_lane"]), int(entry["sweep_threads"])
+
+
+def _solve_ms(solve, args, kw, reps: int = 3) -> float:
+    stream = torch.cuda.current_stream(args[0].device)
+    best = math.inf
+    for _ in range(reps):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record(stream)
+        solve(*args, **kw)
+        b.record(stream)
+        b.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
 
 
 def tune(row_ptr: torch.Tensor, col_idx: torch.Tensor, w: torch.Tensor, mode="max", *,
          candidates=CANDIDATES, save: bool = True) -> dict:
     """Time the sweep for every (sweep_kind, edges_per_lane, sweep_threads)
-    candidate and record the fastest for this graph's signature."""
+    candidate and record the fastest for this graph's signature; (0, 0, 0), the
+    library's default, where that solves the graph in one launch and faster."""
     from .ocm import solve
     lib = _native.load()
     ms = (ctypes.c_double * 4)()
@@ -111,11 +131,21 @@ def tune(row_ptr: torch.Tensor, col_idx: torch.Tensor, w: torch.Tensor, mode="ma
     kind, epl, thr = (int(x) for x in best.split("x"))
     result = {"sweep_kind": kind, "edges_per_lane": epl, "sweep_threads": thr,
               "sweep_ms": timings[best], "timings_ms": timings, "signature": signature(row_ptr)}
+    if row_ptr.numel() - 1 <= ONE_LAUNCH_N:
+        args = (row_ptr, col_idx, w, mode)
+        picked = {"sweep_kind": kind, "edges_per_lane": epl, "sweep_threads": thr}
+        with_it = _solve_ms(solve, args, dict(workspace=ws, **picked))
+        default = _solve_ms(solve, args, dict(workspace=ws))
+        one = solve(*args, workspace=ws).stats["launches"] == 1
+        result["solve_ms"] = default if one and default <= with_it else with_it
+        if one and default <= with_it:
+            result.update(sweep_kind=0, edges_per_lane=0, sweep_threads=0)
     if save:
         with _lock:
             tab = _load_table()
             tab[result["signature"]] = {k: result[k] for k in ("sweep_kind", "edges_per_lane",
-                                                               "sweep_threads", "sweep_ms")}
+                                                               "sweep_threads", "sweep_ms",
+                                                               "solve_ms") if k in result}
             _save_table(tab)
     return result
 
