@@ -235,7 +235,7 @@ static int persistent_grid() {
 static int map_err_bits(int err) {
     if (err & kErrTimeout) return OCM_ERR_TIMEOUT;
     if (err & (kErrInitPolicy | kErrTransit | kErrUnreached)) return OCM_ERR_INVALID_ARG;
-    if (err & (kErrRatioKey | kErrRange)) return OCM_ERR_OVERFLOW;
+    if (err & kErrRatioKey) return OCM_ERR_OVERFLOW;
     if (err & (kErrRowPtr | kErrCol)) return OCM_ERR_BAD_CSR;
     if (err & kErrNoOutEdge) return OCM_ERR_NO_OUT_EDGE;
     if (err & kErrWeightMin) return OCM_ERR_OVERFLOW;
@@ -841,11 +841,11 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
         stats->iterations = (int32_t)(it > fin.small_iters ? it : fin.small_iters);
         stats->cycles = h.res_cycles;
         stats->detect_rounds = fin.rounds_detect;
-        stats->value_rounds = fin.rounds_value;
+        stats->value_rounds = 0;
         stats->switched = h.switched_total;
         stats->launches = launches;
         stats->detect_items = fin.items_detect;
-        stats->value_items = fin.items_value;
+        stats->value_items = 0;
         stats->graph_loop = slot >= 0 ? 1 : 0;
         stats->rebuild_levels = fin.connect_levels;
         stats->batch_small_graphs = fin.small_total;

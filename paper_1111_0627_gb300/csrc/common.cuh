@@ -109,14 +109,12 @@ struct Ctrl {
     int nrep;             // number of policy cycles (roots)
     int maxabsw;          // max |w| over all edges
     int ncand;            // cycle-extraction candidates
-    int rounds_detect;    // jump rounds that had work (cycle detection)
-    int rounds_value;     // jump rounds that had work (value propagation)
-    long long items_detect;   // worklist items processed, all detect rounds
-    long long items_value;    // worklist items processed, all value rounds
+    int rounds_detect;    // one-level evaluations; two-level: rounds on the exits' graph;
+                          //     SCC searches: levels
+    long long items_detect;   // vertices evaluated, all iterations
     unsigned long long best;  // packed (rank, INT_MAX - root) of the best cycle
     GridBar bar[2];           // grid barriers: [0] evaluation (and the SCC kernels), [1] rebuild
-    int pending[3];           // detect: rotating per-round counts of unfinished vertices
-    int pendv[3];             // values: the same
+    int pending[3];           // SCC searches: rotating counters of the backward frontier
     int cls_cnt[8];           // improvement sweep: vertices per degree class (then heavy)
     int cls_off[8];           // start of each class in the class list
     int heavy_edges;          // improvement sweep: edges of all heavy vertices
@@ -239,7 +237,6 @@ enum : int {
     kErrTransit = 1024,   // a transit time below 1
     kErrRatioKey = 2048,  // cycle ratio: the exact order keys of the current cycles overflow int64
     kErrUnreached = 4096, // single-lambda rebuild: a vertex cannot reach the chosen cycle
-    kErrRange = 16384,    // the exactness bound of the weights (solve by one team)
     kErrConnect = 8192,   // single-lambda rebuild: inconsistent state (no chosen cycle, no edge)
 };
 

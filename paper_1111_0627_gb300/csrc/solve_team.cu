@@ -19,6 +19,14 @@
 namespace ocm {
 
 constexpr int kChainLen = 48;   // critical cycles walked by one thread
+// Graphs solved by one team: up to kTeamSolveN vertices with 8 edges each on
+// average (the sweep gives a vertex of up to 32 edges one thread), by one block
+// up to kTeamBlockN.
+constexpr int kTeamSolveN = 16384;
+constexpr int kTeamBlockN = 1024;
+static_assert(2LL * kTeamSolveN * kTeamSolveN < (1LL << 62 >> 31), "values and keys stay exact");
+static_assert((kTeamBlockN / 32 * 4 + 15) / 16 * 16 + 16 * kTeamBlockN <= kTeamBytes,
+              "one block's states fit in its shared memory");
 
 // The checks of check_row_ptr_kernel; also notes vertices of more than
 // kHeavyEdges edges (Ctrl::team_off).
@@ -178,22 +186,15 @@ solve_team_kernel(const int *__restrict__ row_ptr, const int *__restrict__ col,
         tm.sync();   // (the first block's shared memory stays until all are done)
         return;
     }
-    // the exactness bound, 2 n^2 max|w| < 2^62 (n below 2^20)
-    if ((unsigned __int128)(2LL * n * n) * (unsigned)load_volatile(&c->maxabsw) >=
-        ((unsigned __int128)1 << 62)) {
-        if (tm.tid == 0) c->err = kErrRange;
-        tm.sync();
-        return;
-    }
+    // (the exactness bound, 2 n^2 max|w| < 2^62, holds up to kTeamSolveN vertices;
+    // one block's states are in shared memory, see launch_solve_team)
     bool in_shared;
     const TeamGraph g = team_place<C>(s_dyn, row_ptr, col, w, sign, 0, n, ws, room, &in_shared);
     int it = 0;
     long long switched = 0;
     bool capped = false;
     const bool ok =
-        C == 1 && in_shared
-            ? team_iterate<C, C == 1>(tm, g, init != nullptr, max_iters, &it, &switched, &capped)
-            : team_iterate<C, false>(tm, g, init != nullptr, max_iters, &it, &switched, &capped);
+        team_iterate<C, C == 1>(tm, g, init != nullptr, max_iters, &it, &switched, &capped);
     if (tm.tid == 0 && capped) c->not_converged = 1;
     if (ok) {
         const unsigned long long packed = *reinterpret_cast<volatile unsigned long long *>(g.best);
@@ -216,9 +217,6 @@ solve_team_kernel(const int *__restrict__ row_ptr, const int *__restrict__ col,
     tm.sync();
 }
 
-// Graphs solved by one team: up to kTeamSolveN vertices with 8 edges each on
-// average (the sweep gives a vertex of up to 32 edges one thread).
-constexpr int kTeamSolveN = 16384;
 bool team_solves(int n, int m) { return n <= kTeamSolveN && m <= 8LL * n + 1024; }
 
 namespace {
@@ -262,7 +260,7 @@ int launch_solve_team(const int *row_ptr, const int *col, const int *w, int sign
     if (n <= 512)
         return launch_team<1>(256, kTeamBytes, row_ptr, col, w, sign, n, m, init, max_iters,
                               cycle_out, ws, st);
-    if (n <= 1024)
+    if (n <= kTeamBlockN)
         return launch_team<1>(1024, kTeamBytes, row_ptr, col, w, sign, n, m, init, max_iters,
                               cycle_out, ws, st);
     if (n <= 4096)

@@ -49,7 +49,6 @@ struct TeamShared {
     int sum[3];
     int nrep;
     int task;
-    int K;
 };
 
 template <int C>
