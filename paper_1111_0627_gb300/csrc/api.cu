@@ -693,7 +693,7 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
                                   (unsigned long long)nmax * (unsigned)h.maxabsw;
         if (ratio) bound *= 2 * (unsigned __int128)(unsigned)h.maxt;
         if (bound >= ((unsigned __int128)1 << 62)) return OCM_ERR_OVERFLOW;
-        if (ratio && (unsigned long long)nmax * (unsigned)h.maxt > 0x7fffffffULL)
+        if (ratio && (unsigned long long)nmax * (unsigned)h.maxt > (unsigned long long)kMaxPathTime)
             return OCM_ERR_OVERFLOW;
     }
     const long long N2 = nmax * nmax;

@@ -257,7 +257,9 @@ struct Workspace {
     int *cyc_rank;
     int *cid_of_root;
     unsigned *done;       // bitmap: extraction scratch
-    int *cyc_tag;         // [n] one-level: tag of the evaluation that marked the cycle v is on (0: none)
+    int *cyc_tag;         // [n] whole grid, one-level: tag of the evaluation that marked the cycle
+                          //     v is on (0: none); teams (team.cuh): 1 + the root of the cycle
+                          //     that tagged v last
     unsigned *rec_dirty;  // bitmap: the last record pass changed v's record (Ctrl::dirty_on)
     unsigned *need_blk;   // bitmap over blocks of kClassifyBlock vertices: some target of
                           //     the block's edges lies in a block with a changed record
@@ -289,10 +291,12 @@ struct Workspace {
     int *tpi;             // [n] transit time of the policy edge
     long long *jt[2];     // [n] value jumping: transit time of the path from v to J
     long long *recp;      // [n] numerator p of the ratio of v's cycle (gathered by the sweep)
-    int *root_mark;       // [n] one-level: 2 * (tag of the evaluation that listed the root) + 1
-                          //     while its cycle is marked (all its vertices have its cyc_tag,
-                          //     none switched since); two-level evaluation:
-                          //     evaluation stamp of a root found on the node graph
+    int *root_mark;       // [n] whole grid, one-level: 2 * (tag of the evaluation that listed the
+                          //     root) + 1 while its cycle is marked (all its vertices have its
+                          //     cyc_tag, none switched since); two-level evaluation: evaluation
+                          //     stamp of a root found on the node graph; teams: kRootOld to
+                          //     kRootSeed (team.cuh).  A solve's vertices are marked in one of
+                          //     these ways only: a batch's graphs go to a team or to the union.
     int2 *chunk_info;     // [n / 1024 + 2] chunked local pass, per block range: (status, exits)
     // one-level evaluation: jls[k & 1] is the value buffer of evaluation k, and
     // whatever changes a policy edge stores the vertex's one step {succ, 1,
@@ -325,8 +329,12 @@ __device__ __forceinline__ void store_step(const Workspace &ws, int next_eval, i
     }
 }
 
-// Transit time of a path: below 2^31, under the tag of the evaluation that
-// stored it.
+// Transit time of a path, under the tag of the evaluation that stored it: the
+// low half holds every time up to kMaxPathTime, the limit that a solve with
+// transit times checks n max t against before its first evaluation.  (A walk that
+// goes round a new cycle may pass it; its time is then added up again from 0.)
+constexpr long long kMaxPathTime = 0x7fffffff;
+static_assert(kMaxPathTime <= 0xffffffffLL, "a path's time fits beside its tag");
 __device__ __forceinline__ long long path_time(long long tagged) {
     return tagged & 0xffffffffLL;
 }

@@ -709,7 +709,7 @@ walk_kernel(int n, Workspace ws, BatchState bs) {
         }
         int cur = v, len = 0;
         long long S = 0;
-        unsigned T = 0;          // (n max t < 2^31)
+        unsigned T = 0;          // (see kMaxPathTime)
         int total = 0, found = 0;
         unsigned open;           // lanes still walking
         for (;;) {

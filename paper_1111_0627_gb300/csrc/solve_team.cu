@@ -25,8 +25,7 @@ constexpr int kChainLen = 48;   // critical cycles walked by one thread
 constexpr int kTeamSolveN = 16384;
 constexpr int kTeamBlockN = 1024;
 static_assert(2LL * kTeamSolveN * kTeamSolveN < (1LL << 62 >> 31), "values and keys stay exact");
-static_assert((kTeamBlockN / 32 * 4 + 15) / 16 * 16 + 16 * kTeamBlockN <= kTeamBytes,
-              "one block's states fit in its shared memory");
+static_assert(kTeamBlockN <= kTeamSharedN, "one block's states fit in its shared memory");
 
 // The checks of check_row_ptr_kernel; also notes vertices of more than
 // kHeavyEdges edges (Ctrl::team_off).

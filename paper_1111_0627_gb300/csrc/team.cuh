@@ -22,12 +22,18 @@ constexpr int kTeamThreads = 1024;   // largest block
 constexpr int kSU = 4;   // vertices per thread per pass of a jump round (64 registers)
 // Dynamic shared memory of a team's block: the frontier bitmap, then the policy
 // states and in their place, once the cycles are known, the records (16 bytes a
-// vertex: graphs of up to 12,190 vertices), or the bitmaps of the jump rounds.
+// vertex), or the bitmaps of the jump rounds.
 constexpr int kTeamBytes = 196608;
+constexpr int team_bitmap_bytes(int n) { return ((n + 31) / 32 * 4 + 15) / 16 * 16; }
+constexpr int kTeamSharedN = 12192;   // largest graph whose states fit beside the bitmap
+static_assert(team_bitmap_bytes(kTeamSharedN) + 16 * kTeamSharedN <= kTeamBytes &&
+                  team_bitmap_bytes(kTeamSharedN + 1) + 16 * (kTeamSharedN + 1) > kTeamBytes,
+              "kTeamSharedN");
 
 // Evaluation by walks (team_walk): steps between two published parts and between
-// two looks for a new cycle, the most steps of a walk and of a sample, new cycles a warp looks for, and the
-// number of detection rounds up to which the policy counts as shallow enough.
+// two looks for a new cycle, the most steps of a walk and of a sample, new cycles
+// a warp looks for, and the number of detection rounds up to which the policy
+// counts as shallow enough.
 constexpr int kTeamPart = 8;
 constexpr int kTeamTight = 32;
 constexpr int kTeamSteps = 256;
@@ -833,13 +839,13 @@ static __device__ __forceinline__ TeamGraph team_place(unsigned char *dyn, const
                 nullptr, nullptr, reinterpret_cast<unsigned long long *>(ws.recp + v0), ws};
     *in_shared = false;
     const long long nw = (n + 31) / 32;
-    const long long d = ((C == 1 ? nw : 0) * 4 + 15) / 16 * 16;   // the frontier bitmap
+    const long long d = team_bitmap_bytes(n);   // the frontier bitmap
     if (C > 1) {
         g.dirty = reinterpret_cast<unsigned *>(ws.list[1] + v0);
     } else if (d <= room) {
         g.dirty = reinterpret_cast<unsigned *>(dyn);
         if (d + 12 * nw <= room) g.bits = reinterpret_cast<unsigned *>(dyn + d);
-        if (d + 16LL * n <= room) {
+        if (n <= kTeamSharedN) {
             *in_shared = true;
             g.st = reinterpret_cast<JLS *>(dyn + d);
             g.rec = reinterpret_cast<Rec *>(g.st);
