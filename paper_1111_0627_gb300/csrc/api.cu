@@ -724,8 +724,9 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
     if (bs) {
         const int small_n = opt ? opt->batch_small_vertices : 0;   // 0: automatic
         if (small_n >= 0 && !ratio && !outputs) {
-            const int k = launch_batch_small(row_ptr, col_idx, w, sign, small_n, n, h.max_ng, max_iters,
-                                             opt && opt->init_policy ? 1 : 0, b.small_queue, ws, b, st);
+            const int k = launch_batch_small(row_ptr, col_idx, w, sign, small_n, n, h.max_ng,
+                                             max_iters, opt && opt->init_policy ? 1 : 0,
+                                             b.small_queue, ws, b, st);
             if (k < 0) return OCM_ERR_CUDA;
             launches += k;
         }

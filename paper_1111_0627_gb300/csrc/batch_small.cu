@@ -200,7 +200,8 @@ int launch_batch_small(const int *row_ptr, const int *col, const int *w, int sig
     }
     int big_bucket = kBigMinBucket;
     while (big_bucket < 31 && (1LL << big_bucket) < N / (6LL * cached_blocks)) ++big_bucket;
-    const bool has_big = cached_clusters > 0 && big_bucket < 31 && max_ng >= (1 << big_bucket) && max_n >= (1 << big_bucket);
+    const bool has_big = cached_clusters > 0 && big_bucket < 31 && max_ng >= (1 << big_bucket) &&
+                         max_n >= (1 << big_bucket);
     int gb = (bs.G + kThreads - 1) / kThreads;
     if (gb > 1024) gb = 1024;
     prof_begin(kProfEvaluate, st);

@@ -320,6 +320,46 @@ __device__ __forceinline__ void unmark_cycle(const Workspace &ws, int F, int v) 
     }
 }
 
+// Single-copy atomic 16-byte accesses of a policy state that others write and
+// read at the same time (the walks): relaxed, loads through L1; SM: in shared
+// memory.
+template <bool SM>
+__device__ __forceinline__ JLS load_state(const JLS *p) {
+    unsigned long long a, b;
+    if (SM)
+        asm volatile("{ .reg .b128 t; ld.relaxed.cta.shared.b128 t, [%2]; mov.b128 {%0, %1}, t; }"
+                     : "=l"(a), "=l"(b) : "r"((unsigned)__cvta_generic_to_shared(p)) : "memory");
+    else
+        asm volatile("{ .reg .b128 t; ld.relaxed.cta.global.b128 t, [%2]; mov.b128 {%0, %1}, t; }"
+                     : "=l"(a), "=l"(b) : "l"(p) : "memory");
+    return JLS{(int)(unsigned)a, (int)(unsigned)(a >> 32), (long long)b};
+}
+
+template <bool SM>
+__device__ __forceinline__ void store_state(JLS *p, const JLS &s) {
+    const unsigned long long a = (unsigned)s.J | ((unsigned long long)(unsigned)s.len << 32);
+    if (SM)
+        asm volatile("{ .reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.cta.shared.b128 [%0], t; }"
+                     :: "r"((unsigned)__cvta_generic_to_shared(p)), "l"(a),
+                        "l"((unsigned long long)s.S) : "memory");
+    else
+        asm volatile("{ .reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.gpu.global.b128 [%0], t; }"
+                     :: "l"(p), "l"(a), "l"((unsigned long long)s.S) : "memory");
+}
+
+// A short critical cycle: one thread follows the policy from its root r, a
+// microsecond for two or three edges.  The candidates and the lifting take 8
+// launches and 50-80 us (2^20 vertices), most solves' cycles have 2-20 edges.
+constexpr int kChainLen = 48;
+__device__ __forceinline__ void follow_cycle(const Workspace &ws, int r, int L, int *cycle_out) {
+    int y = r;
+    for (int k = 0; k < L; ++k) {
+        cycle_out[k] = ws.pi[y];
+        y = ws.succ[y];
+    }
+    ws.ctrl->cnt[0] = y == r ? L : 0;
+}
+
 // Policy switch of v for the next evaluation's value buffer (Workspace::walk).
 __device__ __forceinline__ void store_step(const Workspace &ws, int next_eval, int v, int succ,
                                            int weight) {

@@ -597,13 +597,10 @@ static __device__ void evaluate_tail(int n, long long N2, int F, const Workspace
 // 100 to 135 steps deep at n = 2^20: 160 us a walk without published parts, 48
 // with; 200 to 400 steps deep at n = 2.4 M (a random digraph's giant component):
 // walks failed after 2.1 ms and an evaluation took 600 us of jump rounds, 125 with.
-// Publishing from 24 steps on gained the random graphs another 4% and cost the
-// product graphs up to 8%, whose small new cycles are then left to the jump
-// rounds; a limit of 64 steps left too much open (13.7 -> 9.1 ms a solve with 128,
-// 12 ms with 64), and reading past L1 after 16 or 32 steps, to see newer parts,
-// took 10-25% longer.  Reading
-// the states past L1 took 220-360 us, and giving each lane its next vertex as
-// soon as it was done (more divergence) 100-300 us.
+// Published parts from 24 steps on cost the product graphs up to 8%, whose small
+// new cycles are then left to the jump rounds; a limit of 64 steps for 128 left
+// too much open (12 ms a solve for 9.1).  Reading the states past L1 took 220-360
+// us a launch.
 // ---------------------------------------------------------------------------
 constexpr int kWalkThreads = 256;
 constexpr int kWalkTight = 32;    // steps up to the first look for a cycle
@@ -614,26 +611,13 @@ constexpr int kSampleThreads = 512;         // samples that look for cycles
 constexpr int kSampleSteps = 512;
 constexpr int kWalkCycles = 8;    // new cycles a warp looks for
 
-static __device__ __forceinline__ JLS load_state(const JLS *p) {   // (through L1)
-    unsigned long long a, b;
-    asm volatile("{ .reg .b128 t; ld.relaxed.cta.global.b128 t, [%2]; mov.b128 {%0, %1}, t; }"
-                 : "=l"(a), "=l"(b) : "l"(p) : "memory");
-    return JLS{(int)(unsigned)a, (int)(unsigned)(a >> 32), (long long)b};
-}
-
-static __device__ __forceinline__ void store_state(JLS *p, const JLS &s) {
-    const unsigned long long a = (unsigned)s.J | ((unsigned long long)(unsigned)s.len << 32);
-    asm volatile("{ .reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.gpu.global.b128 [%0], t; }"
-                 :: "l"(p), "l"(a), "l"((unsigned long long)s.S) : "memory");
-}
-
 // Looks for a cycle on the path from cur.  Returns its smallest vertex, now
 // settled and listed, or -1 if the path meets a settled vertex or is too long.
 static __device__ __forceinline__ int walk_find_cycle(int cur, JLS *st, unsigned tag, int limit,
                                                       const Workspace &ws, int *listed) {
     int tort = cur, lam = 0, power = 1, r = -1;
     for (int k = 0; k < limit; ++k) {
-        const JLS s = load_state(&st[cur]);
+        const JLS s = load_state<false>(&st[cur]);
         if (s.J < 0) return -1;
         cur = s.J;
         if (cur == tort) {
@@ -650,7 +634,7 @@ static __device__ __forceinline__ int walk_find_cycle(int cur, JLS *st, unsigned
     int k = 0;
     for (int y = ws.succ[cur]; y != cur && k < limit; y = ws.succ[y], ++k) r = min(r, y);
     if (k >= limit) return -1;
-    store_state(&st[r], JLS{~r, 0, 0});
+    store_state<false>(&st[r], JLS{~r, 0, 0});
     // the first to find it lists the root and marks the cycle
     volatile int *mark = &ws.root_mark[r];
     if ((unsigned)*mark >> 1 != tag &&
@@ -704,7 +688,7 @@ walk_kernel(int n, Workspace ws, BatchState bs) {
         const bool on = v < n && !(bs.G && bs.gconv[bs.gid[v]]);
         JLS s{-1, 0, 0};
         if (on) {
-            s = load_state(&st[v]);
+            s = load_state<false>(&st[v]);
             next[v] = s.J >= 0 ? s : JLS{ws.succ[v], 1, (long long)ws.wpi[v]};
         }
         int cur = v, len = 0;
@@ -720,7 +704,7 @@ walk_kernel(int n, Workspace ws, BatchState bs) {
                     len += s.len;   // (1 unless published)
                     S += s.S;
                     cur = s.J;
-                    s = load_state(&st[cur]);
+                    s = load_state<false>(&st[cur]);
                     if (RATIO && s.J < 0 && s.len > 0) {
                         const long long tt = ws.jt[F][cur];
                         if ((unsigned)(tt >> 32) == tag)
@@ -735,7 +719,7 @@ walk_kernel(int n, Workspace ws, BatchState bs) {
             total += part;
             if (total >= steps) break;
             if (deep) {
-                if (s.J >= 0 && len <= kWalkPublish) store_state(&st[v], JLS{cur, len, S});
+                if (s.J >= 0 && len <= kWalkPublish) store_state<false>(&st[v], JLS{cur, len, S});
                 continue;
             }
             if (total & (total - 1)) continue;   // (looks after 32, 64 and 128 steps)
@@ -750,7 +734,7 @@ walk_kernel(int n, Workspace ws, BatchState bs) {
                     len = 0;
                     S = 0;
                     T = 0;
-                    s = load_state(&st[v]);
+                    s = load_state<false>(&st[v]);
                 }
             }
         }
@@ -776,7 +760,7 @@ walk_kernel(int n, Workspace ws, BatchState bs) {
                 }
             }
             if (RATIO) ws.jt[F][v] = ((long long)tag << 32) | T;
-            store_state(&st[v], f);
+            store_state<false>(&st[v], f);
         }
         if (open) {
             int sofar = 0;
@@ -1618,20 +1602,8 @@ __global__ void extract_reset_kernel(Workspace ws) {
     ws.ctrl->walk_ok = 0;
 }
 
-// A short critical cycle: one thread follows the policy from its root, a
-// microsecond for two or three edges.  The candidates and the lifting take 8
-// launches and 50-80 us (2^20 vertices), most solves' cycles have 2-20 edges.
-constexpr int kChainLen = 48;
-
 __global__ void extract_chain_kernel(int L, Workspace ws, int *cycle_out) {
-    Ctrl *c = ws.ctrl;
-    const int r = c->res_root;
-    int y = r;
-    for (int k = 0; k < L; ++k) {
-        cycle_out[k] = ws.pi[y];
-        y = ws.succ[y];
-    }
-    c->cnt[0] = y == r ? L : 0;
+    follow_cycle(ws, ws.ctrl->res_root, L, cycle_out);
 }
 
 // Extracts the critical cycle (root and length already in ctrl->res_*);

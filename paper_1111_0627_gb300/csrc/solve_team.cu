@@ -18,7 +18,6 @@
 
 namespace ocm {
 
-constexpr int kChainLen = 48;   // critical cycles walked by one thread
 // Graphs solved by one team: up to kTeamSolveN vertices with 8 edges each on
 // average (the sweep gives a vertex of up to 32 edges one thread), by one block
 // up to kTeamBlockN.
@@ -130,14 +129,7 @@ static __device__ void team_extract(Team<C> &tm, const TeamGraph &g, int r, int 
     const Workspace &ws = g.ws;
     const int n = g.n;
     if (L <= kChainLen) {
-        if (tm.tid == 0) {
-            int y = r;
-            for (int k = 0; k < L; ++k) {
-                cycle_out[k] = ws.pi[y];
-                y = ws.succ[y];
-            }
-            ws.ctrl->cnt[0] = y == r ? L : 0;
-        }
+        if (tm.tid == 0) follow_cycle(ws, r, L, cycle_out);
         return;
     }
     int *cur = ws.aprev, *J = reinterpret_cast<int *>(ws.jm[0]), *J2 = reinterpret_cast<int *>(ws.jm[1]);

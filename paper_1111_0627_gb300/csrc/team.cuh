@@ -100,31 +100,6 @@ struct Team {
     }
 };
 
-// Single-copy atomic 16-byte accesses of a policy state; SM: in shared memory.
-template <bool SM>
-static __device__ __forceinline__ JLS team_load(const JLS *p) {
-    unsigned long long a, b;
-    if (SM)
-        asm volatile("{ .reg .b128 t; ld.relaxed.cta.shared.b128 t, [%2]; mov.b128 {%0, %1}, t; }"
-                     : "=l"(a), "=l"(b) : "r"((unsigned)__cvta_generic_to_shared(p)) : "memory");
-    else
-        asm volatile("{ .reg .b128 t; ld.relaxed.cta.global.b128 t, [%2]; mov.b128 {%0, %1}, t; }"
-                     : "=l"(a), "=l"(b) : "l"(p) : "memory");
-    return JLS{(int)(unsigned)a, (int)(unsigned)(a >> 32), (long long)b};
-}
-
-template <bool SM>
-static __device__ __forceinline__ void team_store(JLS *p, const JLS &s) {
-    const unsigned long long a = (unsigned)s.J | ((unsigned long long)(unsigned)s.len << 32);
-    if (SM)
-        asm volatile("{ .reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.cta.shared.b128 [%0], t; }"
-                     :: "r"((unsigned)__cvta_generic_to_shared(p)), "l"(a),
-                        "l"((unsigned long long)s.S) : "memory");
-    else
-        asm volatile("{ .reg .b128 t; mov.b128 t, {%1, %2}; st.relaxed.gpu.global.b128 [%0], t; }"
-                     :: "l"(p), "l"(a), "l"((unsigned long long)s.S) : "memory");
-}
-
 // The graph a team works on.  st, rec and old are indexed by vertex - v0.
 struct TeamGraph {
     const int *row_ptr, *col, *w;
@@ -233,7 +208,7 @@ static __device__ __forceinline__ int team_seed(Team<C> &tm, const TeamGraph &g,
     int cur = v, tort = v, lam = 0, power = 1, len = 0;
     long long S = 0;
     bool cycle = false, first = false;
-    JLS s = team_load<SM>(&st[cur]);
+    JLS s = load_state<SM>(&st[cur]);
     for (int k = 0; k < kTeamSeedSteps && s.J >= 0; ++k) {
         len += s.len;
         S += s.S;
@@ -247,16 +222,16 @@ static __device__ __forceinline__ int team_seed(Team<C> &tm, const TeamGraph &g,
             power <<= 1;
             lam = 0;
         }
-        s = team_load<SM>(&st[cur]);
+        s = load_state<SM>(&st[cur]);
     }
     if (cycle) team_list_cycle<C>(tm, g, cur, kTeamSeedSteps, &first);
-    else if (s.J < 0 && len > 0) team_store<SM>(&st[v], JLS{s.J, len + s.len, S + s.S});
+    else if (s.J < 0 && len > 0) store_state<SM>(&st[v], JLS{s.J, len + s.len, S + s.S});
     const int fresh = tm.sum(first);
     const int seeded = kept + fresh;
     if (fresh) {
         for (int k = kept + tm.tid; k < seeded; k += tm.W) {
             const int r = ws.cyc_root[g.v0 + k];
-            team_store<SM>(&st[r], JLS{~r, 0, 0});
+            store_state<SM>(&st[r], JLS{~r, 0, 0});
             ws.root_mark[r] = kRootOld;
         }
         tm.sync();
@@ -285,7 +260,7 @@ static __device__ __forceinline__ int team_walk(Team<C> &tm, const TeamGraph &g,
         const int v = base + lane;
         const bool on = v < v1;
         JLS s{-1, 0, 0};
-        if (on) s = team_load<SM>(&st[v]);
+        if (on) s = load_state<SM>(&st[v]);
         int cur = v, len = 0;
         long long S = 0;
         int total = 0, found = 0;
@@ -297,14 +272,14 @@ static __device__ __forceinline__ int team_walk(Team<C> &tm, const TeamGraph &g,
                     len += s.len;
                     S += s.S;
                     cur = s.J;
-                    s = team_load<SM>(&st[cur]);
+                    s = load_state<SM>(&st[cur]);
                 }
             }
             open = __ballot_sync(0xffffffffu, s.J >= 0);
             if (!open) break;
             total += kTeamPart;
             if (total >= kTeamSteps) break;
-            if (s.J >= 0 && len <= kTeamPublish) team_store<SM>(&st[v], JLS{cur, len, S});
+            if (s.J >= 0 && len <= kTeamPublish) store_state<SM>(&st[v], JLS{cur, len, S});
             if (total % kTeamTight) continue;
             int r = -1;
             if (lane == __ffs(open) - 1) {
@@ -322,7 +297,7 @@ static __device__ __forceinline__ int team_walk(Team<C> &tm, const TeamGraph &g,
                         power <<= 1;
                         lam = 0;
                     }
-                    if (team_load<SM>(&st[y]).J < 0) break;
+                    if (load_state<SM>(&st[y]).J < 0) break;
                 }
                 if (cycle) r = team_list_cycle<C>(tm, g, y, 2 * total, &first);
                 if (r >= 0 && first) {
@@ -331,9 +306,9 @@ static __device__ __forceinline__ int team_walk(Team<C> &tm, const TeamGraph &g,
                     // may go round the cycle without ever stopping at the root;
                     // nothing is settled by it before the root is, here)
                     for (y = ws.succ[r]; y != r; y = ws.succ[y])
-                        team_store<SM>(&st[y], JLS{ws.succ[y], 1, (long long)ws.wpi[y]});
+                        store_state<SM>(&st[y], JLS{ws.succ[y], 1, (long long)ws.wpi[y]});
                     __threadfence();   // (before anything that follows from the root)
-                    team_store<SM>(&st[r], JLS{~r, 0, 0});
+                    store_state<SM>(&st[r], JLS{~r, 0, 0});
                 }
             }
             r = __reduce_max_sync(0xffffffffu, r);
@@ -364,7 +339,7 @@ static __device__ __forceinline__ int team_walk(Team<C> &tm, const TeamGraph &g,
                 if (y == root) f = JLS{~root, k, Sy};
                 __threadfence();   // (after the cycle's states were put back, above)
             }
-            team_store<SM>(&st[v], f);
+            store_state<SM>(&st[v], f);
         }
         left += on && s.J >= 0;
     }
@@ -503,7 +478,10 @@ static __device__ int team_jump(Team<C> &tm, const TeamGraph &g) {
         for (int base = tm.tid; base < nk; base += kSU * Wt) {
             JLS sj[kSU], tj[kSU];
 #pragma unroll
-            for (int u = 0; u < kSU; ++u) { const int d = base + u * Wt; sj[u] = d < nk ? A[d] : JLS{-1, 0, 0}; }
+            for (int u = 0; u < kSU; ++u) {
+                const int d = base + u * Wt;
+                sj[u] = d < nk ? A[d] : JLS{-1, 0, 0};
+            }
 #pragma unroll
             for (int u = 0; u < kSU; ++u) if (sj[u].J >= 0) tj[u] = A[sj[u].J];
 #pragma unroll
