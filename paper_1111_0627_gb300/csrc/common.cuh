@@ -173,8 +173,10 @@ struct Ctrl {
     int walk_fail;            // walks were dropped before in this solve
     int walk_tries;           // how often they left too much,
     int walk_pause;           // and the evaluations that jump before they are tried again
-    int carry;                // the next evaluation jumps, and finds the states of this one in
-                              // its buffer where no switch has put a step
+    int jump_next;            // after jump rounds: so does the next evaluation,
+    int carry;                // and finds the states of this one in its buffer where no switch
+                              // has put a step
+    int few_switch;           // the last sweep left most paths without a switch
     int walk_deep;            // the next walks publish their parts (deep policies, evaluate.cu)
     unsigned long long depth_sum;   // path lengths of the policy just evaluated, of every eighth
     int depth_cnt;                  // block's vertices: their sum, and how many

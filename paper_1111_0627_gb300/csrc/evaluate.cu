@@ -800,8 +800,10 @@ loop_control_kernel(Workspace ws, BatchState bs, int n, long long max_iters, int
     const int K = c->nrep, iter = c->iter;
     JLS *next = ws.jls[(iter + 1) & 1];
     const int tag = iter + 2;   // of the next evaluation
+    const bool jumped = !c->walk_on || c->walk_left > (n >> kWalkOffShift);
     int kept = 0;
-    if (more && ws.walk && K <= 32) {   // (any policy but the first ones: one warp, no barrier)
+    const bool settle = more && ws.walk && !(jumped && c->jump_next);
+    if (settle && K <= 32) {   // (any policy but the first ones: one warp, no barrier)
         if (warp == 0) {
             const int r = lane < K ? ws.cyc_root[lane] : -1;
             const bool keep = r >= 0 && (ws.root_mark[r] & 1) && !(bs.G && bs.gconv[bs.gid[r]]);
@@ -815,7 +817,7 @@ loop_control_kernel(Workspace ws, BatchState bs, int n, long long max_iters, int
             }
             kept = __popc(m);
         }
-    } else if (more && ws.walk && K <= kSettleRoots) {
+    } else if (settle && K <= kSettleRoots) {
         for (int base = 0; base < K; base += kSampleThreads) {
             const int at = base + (int)threadIdx.x;
             const int r = at < K ? ws.cyc_root[at] : -1;
@@ -856,7 +858,6 @@ loop_control_kernel(Workspace ws, BatchState bs, int n, long long max_iters, int
         c->dirty_on = c->mark;
         c->dirty_cnt = 0;
         c->changed = 0;
-        c->switched = 0;
         // (not at the next evaluation's start: where the walks settled every
         // vertex its blocks pass no barrier before they raise it)
         c->qmax = 0;
@@ -877,12 +878,14 @@ loop_control_kernel(Workspace ws, BatchState bs, int n, long long max_iters, int
             c->walk_fail = 1;
             c->walk_tries = min(c->walk_tries + 1, 20);
         }
+        c->few_switch = c->switched < (n >> 4);
         // (the ratio's sums stay 0)
         c->walk_deep = c->depth_sum > (unsigned long long)kWalkDeep * (unsigned)c->depth_cnt &&
                        (bs.G == 0 || c->active_graphs <= kWalkDeepGraphs);
         c->depth_sum = 0;
         c->depth_cnt = 0;
-        if (!c->walk_on && !c->carry)   // (carry: certain to jump, see evaluate_kernel)
+        c->switched = 0;
+        if (!c->walk_on && !c->jump_next)   // (certain to jump: see evaluate_kernel)
             c->walk_on = !c->walk_fail
                              ? bs.G || K <= kSettleRoots
                              : c->walk_pause == 0 && K <= kSettleRoots &&
@@ -937,9 +940,9 @@ void launch_walk_seed(int n, Workspace ws, cudaStream_t st) {
 // All vertices take part in the detection, whose window minima carry a second
 // bit: a vertex of the window switched.  A vertex without one on its whole path
 // and cycle keeps its state.
-template <bool RATIO>
-static __device__ bool jump_resolve(int n, int F, bool all, bool carry, int max_detect,
-                                    int max_value, const Workspace &ws, const BatchState &bs,
+template <bool RATIO, bool all>
+static __device__ bool jump_resolve(int n, int F, bool carry, int max_detect, int max_value,
+                                    const Workspace &ws, const BatchState &bs,
                                     int *s_cnt, int *rounds) {
     Ctrl *c = ws.ctrl;
     constexpr bool ratio = RATIO;   // optimal cycle ratio: times ride along
@@ -1256,24 +1259,30 @@ evaluate_kernel(int n, long long N2, int max_detect, int max_value, int stall_te
     // What the record pass leaves in the next evaluation's buffer, where the
     // sweep's switches then put their steps: nothing where the walks have put
     // every vertex's step; the steps; or, where the next evaluation is sure to
-    // jump, the final states, which a vertex whose path sees no switch then keeps.
-    // Deep policies change little a step: 300,000 vertices, paths of up to 10,000,
-    // 205 iterations, take 32.5 ms (38.8 with all values found anew and a walk
-    // tried each time); 2,000,000 134 (165).
+    // jump, the final states, which a vertex whose path sees no switch then keeps,
+    // if the last sweep left many such (otherwise nothing: the jump rounds start
+    // from the policy).  Late steps of deep policies change little: 300,000
+    // vertices, paths of up to 10,000, 205 iterations, take 33 ms (38.8 with all
+    // values found anew and a walk tried each time); 2,000,000 137 (165).
     int leave = kLeaveNothing;
     if (all || left > 0) {
         int rounds = 0;
-        if (!jump_resolve<RATIO>(n, F, all, carry, max_detect, max_value, ws, bs, &s_cnt, &rounds))
+        if (!(all ? jump_resolve<RATIO, true>(n, F, carry, max_detect, max_value, ws, bs, &s_cnt,
+                                              &rounds)
+                  : jump_resolve<RATIO, false>(n, F, false, max_detect, max_value, ws, bs, &s_cnt,
+                                               &rounds)))
             return;
         const bool dropped = c->walk_fail || failed;
         const bool stays =
             all && (load_volatile(&c->nrep) > kSettleRoots
                         ? dropped || bs.G == 0
                         : dropped && (rounds > kWalkDeepRounds || walk_pause(c, n) > 0));
-        if (all) leave = stays ? kLeaveStates : kLeaveSteps;
+        const bool keep = stays && c->few_switch;
+        if (all) leave = keep ? kLeaveStates : stays ? kLeaveNothing : kLeaveSteps;
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             c->jump_rounds = rounds;
-            c->carry = stays ? 1 : 0;
+            c->jump_next = stays ? 1 : 0;
+            c->carry = keep ? 1 : 0;
         }
     }
     evaluate_tail<RATIO>(n, N2, F, ws, bs, s_key, leave);

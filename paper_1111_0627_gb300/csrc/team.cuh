@@ -41,6 +41,7 @@ constexpr int kTeamSeedSteps = 512;
 constexpr int kTeamCycles = 8;
 constexpr int kTeamPublish = 1 << 22;   // longest published part (times kTeamSteps: an int)
 constexpr int kTeamWalkRounds = 9;
+constexpr int kTeamFirstRounds = 12;   // (before any was dropped)
 constexpr int kTeamMarkLen = 256;   // longest cycle whose vertices are tagged
 constexpr int kTeamRankSplit = 512;  // cycles from which several threads rank one
 
@@ -54,6 +55,7 @@ static __device__ __forceinline__ unsigned cluster_rank() {
 struct TeamShared {
     int sum[3];
     int nrep;
+    int quit;
     int task;
 };
 
@@ -192,13 +194,19 @@ static __device__ __forceinline__ int team_list_cycle(const Team<C> &tm, const T
 // itself.)
 //   rest: what remains walks to the settled vertices, 4 steps on average.  A
 // walk still open after kTeamPart steps publishes the part it has walked, so that
-// those behind it take it in one step; after kTeamTight one lane of its warp
-// looks for a cycle the samples missed, and a vertex that ends at such a root adds its steps
-// up again, to the first time its path meets it.
+// those behind it take it in one step; after kTeamTight (and twice, four times as
+// many) one lane of its warp looks for a cycle the samples missed, and a vertex
+// that ends at such a root adds its steps up again, to the first time its path
+// meets it.
+//   giving up: one vertex left open sends all to the jump rounds, so the first
+// warp to leave one tells the others.  A cycle of 2,852 in 3,000 vertices, solved
+// by one block: 1.75 ms with every warp walking to the end and looking eight
+// times, 0.59 now, 0.53 with jump rounds alone.
 
 // The seed phase, after which `kept` old roots and the new ones are listed;
 // returns their number, the same in every thread (the shared counter may be
-// raised by those already walking).
+// raised by those already walking), or -1 where an eighth of the samples met
+// neither a settled vertex nor a cycle: too deep to walk.
 template <int C, bool SM>
 static __device__ __forceinline__ int team_seed(Team<C> &tm, const TeamGraph &g, JLS *st,
                                                 int kept) {
@@ -226,7 +234,10 @@ static __device__ __forceinline__ int team_seed(Team<C> &tm, const TeamGraph &g,
     }
     if (cycle) team_list_cycle<C>(tm, g, cur, kTeamSeedSteps, &first);
     else if (s.J < 0 && len > 0) store_state<SM>(&st[v], JLS{s.J, len + s.len, S + s.S});
-    const int fresh = tm.sum(first);
+    // (both counts are at most the team's 16,384 threads)
+    const int both = tm.sum((int)first + ((tm.tid < g.n && !cycle && s.J >= 0) << 16));
+    const int fresh = both & 0xffff;
+    if ((both >> 16) > tm.W >> 3) return -1;
     const int seeded = kept + fresh;
     if (fresh) {
         for (int k = kept + tm.tid; k < seeded; k += tm.W) {
@@ -253,7 +264,9 @@ static __device__ __forceinline__ int team_walk(Team<C> &tm, const TeamGraph &g,
     JLS *st = g.st - g.v0;
     const int v1 = g.v0 + g.n;
     bool first = false;
+    volatile int *quit = &tm.sh->quit;   // a warp gave up
     const int seeded = team_seed<C, SM>(tm, g, st, kept);
+    if (seeded < 0) return g.n;
     const int root0 = seeded > 0 ? ws.cyc_root[g.v0] : -1;
     int left = 0;
     for (int base = g.v0 + tm.tid - lane; base < v1; base += tm.W) {
@@ -280,7 +293,8 @@ static __device__ __forceinline__ int team_walk(Team<C> &tm, const TeamGraph &g,
             total += kTeamPart;
             if (total >= kTeamSteps) break;
             if (s.J >= 0 && len <= kTeamPublish) store_state<SM>(&st[v], JLS{cur, len, S});
-            if (total % kTeamTight) continue;
+            if (total < kTeamTight || (total & (total - 1))) continue;   // (looks after 32, 64, 128)
+            if (__any_sync(0xffffffffu, *quit)) break;   // (the whole warp or none of it)
             int r = -1;
             if (lane == __ffs(open) - 1) {
                 // (policy edges, not states: those may skip ahead)
@@ -342,6 +356,11 @@ static __device__ __forceinline__ int team_walk(Team<C> &tm, const TeamGraph &g,
             store_state<SM>(&st[v], f);
         }
         left += on && s.J >= 0;
+        if (open) {   // (what one leaves open sends all to the jump rounds)
+            *quit = 1;
+            break;
+        }
+        if (C == 1 && __any_sync(0xffffffffu, *quit)) break;
     }
     return tm.sum(left);
 }
@@ -518,10 +537,11 @@ static __device__ int team_jump(Team<C> &tm, const TeamGraph &g) {
     return rounds;
 }
 
-// Whether and how the next evaluation walks.
+// Whether the next evaluation walks (else jump rounds): not for 0, 1, 3, 7 ..
+// evaluations after walks that were dropped, counted from the last that were not.
 struct TeamMode {
-    bool walk;        // walks (else jump rounds)
-    bool failed;      // walks were dropped before
+    bool walk;
+    int tries, pause;
 };
 
 // Policy evaluation: states, cycle table, records {V, rank, q} (with mark: the
@@ -535,6 +555,7 @@ static __device__ bool team_evaluate(Team<C> &tm, const TeamGraph &g, TeamMode &
     const Workspace &ws = g.ws;
     const int n = g.n, v0 = g.v0;
     const int W = tm.W;
+    bool walked = false;
     if (mode.walk) {
         int kept = 0;   // roots whose cycle no switch broke
         for (int base = tm.tid; base < n; base += kSU * W) {
@@ -563,18 +584,22 @@ static __device__ bool team_evaluate(Team<C> &tm, const TeamGraph &g, TeamMode &
                 g.st[i] = s;
             }
         }
-        if (team_walk<C, SM>(tm, g, tm.sum(kept)) > 0) {
-            mode.walk = false;
-            mode.failed = true;
+        if (tm.tid == 0) tm.sh->quit = 0;
+        walked = team_walk<C, SM>(tm, g, tm.sum(kept)) == 0;
+        if (!walked) mode.pause = (1 << mode.tries) - 1;
+        mode.tries = walked ? 0 : min(mode.tries + 1, 20);
+        if (!walked) {
             if (tm.tid == 0) tm.sh->nrep = 0;
             tm.sync();
         }
+    } else if (mode.pause > 0) {
+        --mode.pause;
     }
-    if (!mode.walk) {
+    if (!walked) {
         for (int i = tm.tid; i < n; i += W) ws.root_mark[v0 + i] = 0;
         const int rounds = team_jump<C>(tm, g);
         if (rounds < 0) return false;
-        mode.walk = !mode.failed || rounds <= kTeamWalkRounds;
+        mode.walk = mode.pause == 0 && rounds <= (mode.tries ? kTeamWalkRounds : kTeamFirstRounds);
         // (the next evaluation walks from these cycles' roots)
         if (mode.walk) {
             const int K = *reinterpret_cast<volatile int *>(&tm.sh->nrep);
@@ -840,7 +865,7 @@ static __device__ bool team_iterate(Team<C> &tm, const TeamGraph &g, bool warm,
                                     long long max_iters, int *iters, long long *switched,
                                     bool *capped) {
     const int n = g.n;
-    TeamMode mode{warm, false};
+    TeamMode mode{warm, 0, 0};
     int last_sw = n;
     long long it = 0, total = 0;
     *capped = false;
