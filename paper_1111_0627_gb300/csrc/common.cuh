@@ -172,7 +172,8 @@ struct Ctrl {
     int jump_rounds;
     int walk_fail;            // walks were dropped before in this solve
     int walk_tries;           // how often they left too much,
-    int walk_pause;           // and the evaluations that jump before they are tried again
+    int walk_pause;           // the evaluations that jump before they are tried again,
+    int walk_rounds;          // and the detection rounds of the last that left too much
     int jump_next;            // after jump rounds: so does the next evaluation,
     int carry;                // and finds the states of this one in its buffer where no switch
                               // has put a step

@@ -775,7 +775,9 @@ walk_kernel(int n, Workspace ws, BatchState bs) {
 // this one: see loop_control_kernel.
 static __device__ __forceinline__ int walk_pause(const Ctrl *c, int n) {
     if (c->walk_on)
-        return c->walk_left > (n >> kWalkOffShift) ? (1 << c->walk_tries) - 1 : 0;
+        return c->walk_left <= (n >> kWalkOffShift) || c->walk_tries == 0 ? 0
+               : c->walk_tries == 1                                       ? 2
+                                                                          : 31;
     return max(c->walk_pause - 1, 0);
 }
 
@@ -867,16 +869,19 @@ loop_control_kernel(Workspace ws, BatchState bs, int n, long long max_iters, int
         // cycles than are settled ahead jumps (9.1 ms a solve, 11.5 with a walk
         // tried each time; 5,000 cycles: 4.0 ms jumping, 3.6 walking, 4.9
         // walking with 1,024 settled); a batch, each of whose warps meets one
-        // or two graphs, is tried.  Walks that left too much are tried again
-        // after 0, 1, 3, 7 .. evaluations, counted from the last that did not,
-        // so that a policy that stays too deep pays for few.
+        // or two graphs, is tried.  Walks that left too much are tried again at
+        // once, then after 2, then after every 31 evaluations, counted from the last
+        // that did not, or when the policy has become shallower by a jump round (700,000
+        // vertices of the locality family, 130 steps deep and solved again:
+        // 4.2 ms a solve, 4.6 with a try after 1, 3, 7, 15; 3.5 with jump rounds alone).
         c->walk_pause = walk_pause(c, n);
         if (c->walk_on && c->walk_left <= (n >> kWalkOffShift)) {
             c->walk_tries = 0;
         } else if (c->walk_on) {
             c->walk_on = 0;
             c->walk_fail = 1;
-            c->walk_tries = min(c->walk_tries + 1, 20);
+            c->walk_tries += 1;
+            c->walk_rounds = c->jump_rounds;
         }
         c->few_switch = c->switched < (n >> 4);
         // (the ratio's sums stay 0)
@@ -888,7 +893,8 @@ loop_control_kernel(Workspace ws, BatchState bs, int n, long long max_iters, int
         if (!c->walk_on && !c->jump_next)   // (certain to jump: see evaluate_kernel)
             c->walk_on = !c->walk_fail
                              ? bs.G || K <= kSettleRoots
-                             : c->walk_pause == 0 && K <= kSettleRoots &&
+                             : (c->walk_pause == 0 || c->jump_rounds < c->walk_rounds) &&
+                                   K <= kSettleRoots &&
                                    c->jump_rounds <= (c->walk_deep ? kWalkDeepRounds : kWalkRounds);
         if (more) {
             c->nrep = kept;
@@ -1276,7 +1282,9 @@ evaluate_kernel(int n, long long N2, int max_detect, int max_value, int stall_te
         const bool stays =
             all && (load_volatile(&c->nrep) > kSettleRoots
                         ? dropped || bs.G == 0
-                        : dropped && (rounds > kWalkDeepRounds || walk_pause(c, n) > 0));
+                        : dropped && (rounds > kWalkDeepRounds ||
+                                      (walk_pause(c, n) > 0 &&
+                                       (failed || rounds >= c->walk_rounds))));
         const bool keep = stays && c->few_switch;
         if (all) leave = keep ? kLeaveStates : stays ? kLeaveNothing : kLeaveSteps;
         if (blockIdx.x == 0 && threadIdx.x == 0) {
