@@ -758,7 +758,7 @@ static int solve_impl(const int32_t *row_ptr, const int32_t *col_idx, const int3
                              (double)h.local_edges >= kLocalEvalMinFraction * (double)m));
     ws.walk = sa.local ? 0 : 1;
     if (ws.walk && !seed) {
-        launch_walk_seed(n, ws, st);
+        launch_walk_seed(n, (double)h.local_edges >= kWalkMaxLocal * (double)m, ws, st);
         launches += 1;
     }
     sa.ws = ws;

@@ -200,6 +200,14 @@ constexpr int kWalkRounds = 9;
 constexpr int kWalkDeep = 48;
 constexpr int kWalkDeepRounds = 12;
 constexpr int kWalkDeepGraphs = 64;  // (of a batch: active graphs at most)
+constexpr int kWalkLongPause = 31;   // evaluations between two tries after failures in a row
+// A graph whose policies are expected to be too deep to walk: this fraction of
+// its edges stays inside the block ranges (a range is n / 152 vertices), so a path
+// takes hundreds of steps to cross them.  Locality family, fraction 0.37 (450,000
+// vertices): walking 4.07 ms a solve, jumping 4.52; 0.39 (500,000): 4.87 and 4.43,
+// 0.59 (10^6): 8.4 and 8.2; solved again from the last policy 3.46 and 3.02, 7.5
+// and 7.1.
+constexpr double kWalkMaxLocal = 0.38;
 // Roots settled ahead of the walks at most: one block does it, 16 rounds of a
 // few gathers at this number.
 constexpr int kSettleRoots = 8192;
@@ -574,7 +582,7 @@ void launch_check_row_ptr(const int *row_ptr, int n, int m, Ctrl *ctrl, cudaStre
 void launch_init_policy(const int *row_ptr, const int *col, const int *w, int sign, int n, int m,
                         const int *init, Workspace ws, const BatchState *bs, cudaStream_t st,
                         int local_R = 0, int count_win = 0, int band_blocks = 1, int seed = 1);
-void launch_walk_seed(int n, Workspace ws, cudaStream_t st);
+void launch_walk_seed(int n, bool jump, Workspace ws, cudaStream_t st);
 int launch_sweep(const int *row_ptr, const int *col, const int *w, int sign, int n,
                  Workspace ws, const int *cls_cnt, int heavy_edges, BatchState bs, int threads,
                  int band_blocks, cudaStream_t st);

@@ -777,7 +777,7 @@ static __device__ __forceinline__ int walk_pause(const Ctrl *c, int n) {
     if (c->walk_on)
         return c->walk_left <= (n >> kWalkOffShift) || c->walk_tries == 0 ? 0
                : c->walk_tries == 1                                       ? 2
-                                                                          : 31;
+                                                                          : kWalkLongPause;
     return max(c->walk_pause - 1, 0);
 }
 
@@ -919,19 +919,28 @@ void launch_loop_control(int n, long long max_iters, Workspace ws, BatchState bs
 }
 
 // The first evaluation's one-step states (when the initial pass left them out).
-__global__ void __launch_bounds__(kThreads) walk_seed_kernel(int n, Workspace ws) {
+// jump: a policy that is expected to be too deep; as after walks that failed
+// several times in a row.
+__global__ void __launch_bounds__(kThreads) walk_seed_kernel(int n, int jump, Workspace ws) {
     const int stride = gridDim.x * blockDim.x;
+    if (jump && blockIdx.x == 0 && threadIdx.x == 0) {
+        Ctrl *c = ws.ctrl;
+        c->walk_on = 0;
+        c->walk_fail = 1;
+        c->walk_tries = 2;
+        c->walk_pause = kWalkLongPause;
+    }
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
         ws.jls[0][v] = JLS{ws.succ[v], 1, (long long)ws.wpi[v]};
         ws.cyc_tag[v] = 0;
     }
 }
 
-void launch_walk_seed(int n, Workspace ws, cudaStream_t st) {
+void launch_walk_seed(int n, bool jump, Workspace ws, cudaStream_t st) {
     int blocks = (n + kThreads - 1) / kThreads;
     if (blocks > 4096) blocks = 4096;
     prof_begin(kProfInit, st);
-    walk_seed_kernel<<<blocks, kThreads, 0, st>>>(n, ws);
+    walk_seed_kernel<<<blocks, kThreads, 0, st>>>(n, jump ? 1 : 0, ws);
     prof_end(kProfInit, st);
 }
 
