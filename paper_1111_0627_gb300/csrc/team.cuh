@@ -36,10 +36,13 @@ static_assert(team_bitmap_bytes(kTeamSharedN) + 16 * kTeamSharedN <= kTeamBytes 
 // counts as shallow enough.
 constexpr int kTeamPart = 8;
 constexpr int kTeamTight = 32;
-constexpr int kTeamSteps = 256;
-constexpr int kTeamSeedSteps = 512;
+// (states in shared memory: jump rounds take 40-80 us there, and so does a walk of
+// some 100 steps with its looks; 1,024 graphs of up to 200,000 vertices, whose
+// states are in global memory, took 79 ms with the smaller limits, 72 with these)
+constexpr int team_steps(bool sm) { return sm ? 128 : 256; }
+constexpr int team_seed_steps(bool sm) { return sm ? 256 : 512; }
 constexpr int kTeamCycles = 8;
-constexpr int kTeamPublish = 1 << 22;   // longest published part (times kTeamSteps: an int)
+constexpr int kTeamPublish = 1 << 22;   // longest published part (times team_steps: an int)
 constexpr int kTeamWalkRounds = 9;
 constexpr int kTeamFirstRounds = 12;   // (before any was dropped)
 constexpr int kTeamMarkLen = 256;   // longest cycle whose vertices are tagged
@@ -217,7 +220,7 @@ static __device__ __forceinline__ int team_seed(Team<C> &tm, const TeamGraph &g,
     long long S = 0;
     bool cycle = false, first = false;
     JLS s = load_state<SM>(&st[cur]);
-    for (int k = 0; k < kTeamSeedSteps && s.J >= 0; ++k) {
+    for (int k = 0; k < team_seed_steps(SM) && s.J >= 0; ++k) {
         len += s.len;
         S += s.S;
         cur = s.J;
@@ -232,7 +235,7 @@ static __device__ __forceinline__ int team_seed(Team<C> &tm, const TeamGraph &g,
         }
         s = load_state<SM>(&st[cur]);
     }
-    if (cycle) team_list_cycle<C>(tm, g, cur, kTeamSeedSteps, &first);
+    if (cycle) team_list_cycle<C>(tm, g, cur, team_seed_steps(SM), &first);
     else if (s.J < 0 && len > 0) store_state<SM>(&st[v], JLS{s.J, len + s.len, S + s.S});
     // (both counts are at most the team's 16,384 threads)
     const int both = tm.sum((int)first + ((tm.tid < g.n && !cycle && s.J >= 0) << 16));
@@ -291,7 +294,7 @@ static __device__ __forceinline__ int team_walk(Team<C> &tm, const TeamGraph &g,
             open = __ballot_sync(0xffffffffu, s.J >= 0);
             if (!open) break;
             total += kTeamPart;
-            if (total >= kTeamSteps) break;
+            if (total >= team_steps(SM)) break;
             if (s.J >= 0 && len <= kTeamPublish) store_state<SM>(&st[v], JLS{cur, len, S});
             if (total < kTeamTight || (total & (total - 1))) continue;   // (looks after 32, 64, 128)
             if (__any_sync(0xffffffffu, *quit)) break;   // (the whole warp or none of it)
