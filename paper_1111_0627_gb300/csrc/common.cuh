@@ -311,8 +311,9 @@ struct Workspace {
     int2 *chunk_info;     // [n / 1024 + 2] chunked local pass, per block range: (status, exits)
     // one-level evaluation: jls[k & 1] is the value buffer of evaluation k, and
     // whatever changes a policy edge stores the vertex's one step {succ, 1,
-    // weight} in the next evaluation's buffer (0 in the two-level form, which
-    // starts from succ and wpi)
+    // weight} in the next evaluation's buffer, where every other vertex has its
+    // step or, before jump rounds, possibly its last state (Ctrl::carry).  (0 in
+    // the two-level form, which starts from succ and wpi)
     int walk;
     Ctrl *ctrl;
 };

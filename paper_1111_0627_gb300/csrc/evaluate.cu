@@ -33,16 +33,15 @@
 //
 // Where the policy graph is shallow, walk_kernel resolves the vertices before
 // this kernel runs, and the jump rounds of detect and values serve what it
-// leaves (see Walks below).
+// leaves (see Walks below).  Where one evaluation after the other jumps, a vertex
+// whose path and cycle saw no switch keeps its state (jump_resolve).
 //
 // Execution: one cooperative launch (all CTAs co-resident) runs every phase;
 // rounds are separated by a grid barrier whose waits are bounded (on expiry
-// the kernel records kErrTimeout and returns).  Rounds are dense over the
-// vertices (coalesced own-state access, no worklist atomics); a bitmap marks
-// vertices that are finished and whose final state sits in both jump buffers,
-// so they cost nothing in later rounds.  A round writes only the buffer it
-// does not read; a vertex resolved in round k copies its final state into the
-// other buffer in round k+1.
+// the kernel records kErrTimeout and returns).  Every block works through the
+// list of its own range's unfinished vertices, so that finished ones cost nothing
+// in later rounds.  A round writes only the buffer it does not read; a vertex
+// resolved in round k copies its final state into the other buffer in round k+1.
 #include <climits>
 
 #include "common.cuh"
