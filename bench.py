@@ -213,9 +213,9 @@ TRAFFIC = {
     # n = 2^23 capture (launches from the middle of a solve, mean; the
     # evaluation's two launches, local_chunk_kernel + evaluate_local_kernel;
     # the sweep's full instance) x 4
-    ("locality32m", "evaluate"): (4 * (0.067920e9 + 0.174084e9 + 0.191438e9 + 0.133894e9),
-                                  "d516308f4f43a93f"),
-    ("locality32m", "sweep"): (4 * (0.862757e9 + 0.122895e9), "7327f46a463627d3"),
+    ("locality32m", "evaluate"): (4 * (0.067974e9 + 0.173948e9 + 0.192057e9 + 0.135132e9),
+                                  "483c32b7423ba4b4"),
+    ("locality32m", "sweep"): (4 * (0.829662e9 + 0.088263e9), "327c433a5699921e"),
 }
 
 
