@@ -363,7 +363,6 @@ static __device__ __forceinline__ int team_walk(Team<C> &tm, const TeamGraph &g,
             *quit = 1;
             break;
         }
-        if (C == 1 && __any_sync(0xffffffffu, *quit)) break;
     }
     return tm.sum(left);
 }
